@@ -131,7 +131,6 @@ DevTree dev_tree(const neuvv_tree *t) {
   d.T = t->info.T;
   d.K = t->info.K;
   d.rec_stride = t->info.rec_stride;
-  d.smem_nodes = 0;
   d.bricks = t->bricks;
   d.brick_level = t->brick_level;
   d.brick_first = t->brick_first;

@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(256) compose_kernel(const __grid_constant__ Co
           float u = fmodf(t * period + pp.toff, period);
           if (u < 0.f) u += period;
           // world distance = t_base + (local distance) * |d| / |dl|
-          integrate_walk<KP, DEG, E, false>(tr, nullptr, w, dn, u, a.t_stop, a.act, t_base, dist_scale, r);
+          integrate_walk<KP, DEG, E>(tr, w, dn, u, a.t_stop, a.act, t_base, dist_scale, r);
         }
         Lc[j][0] = pp.tint[0] * r.C[0];
         Lc[j][1] = pp.tint[1] * r.C[1];

@@ -42,7 +42,7 @@ struct DevTree {
   float bmin[3], bmax[3];
   float scale[3];         // 2^depth / (bmax - bmin)
   float hh_norm[16];      // Abar_{n,l} at [4n + l]
-  int depth, T, K, rec_stride, smem_nodes;
+  int depth, T, K, rec_stride;
   // Bricks: for each internal node at brick_level (nodes brick_first ..
   // brick_first + brick_count - 1), a dense table over its finest cells of
   // (level << 28 | leaf id), an id from kBrickBoxBase up for empty: the node
@@ -101,18 +101,36 @@ __device__ __forceinline__ void raise_status(const DevTree &tr, uint32_t bit) {
 //     cell boundary goes to the side the ray moves towards), clamped to the
 //     node just left.
 // Every distance is along the unit direction, in world units.
+//
+// Mirrored axes.  The walk is bound by the instructions and the dependent
+// chain of its step, so an axis on which the ray moves towards lower
+// coordinates is kept mirrored: position -p, cell ~c = -c - 1, direction and
+// inverse positive.  Negation is exact, so every product, sum and rounding is
+// that of the unmirrored walk, and one code path serves both directions: the
+// ray leaves a box across its upper plane F, the cell behind it is F, and the
+// cell of a point is its floor (for a mirrored axis that is ceil(p) - 1).
+// Only a box's extents ahead of the ray are ever decoded.  Cells are held with
+// the bits of 1.5 * 2^23 added, so that a cell or plane read as a float and
+// reduced by 1.5 * 2^23 is its exact FP32 value, and the floor of p is the
+// bits of p + 1.5 * 2^23 rounded down: no conversion instruction in the step.
 // ---------------------------------------------------------------------------
+constexpr int kMagicBits = 0x4B400000;      // 1.5 * 2^23 as bits ...
+constexpr float kMagic = 12582912.f;        // ... and as a value (|cell| < 2^22)
+constexpr int kBrickShift = 3;              // a brick holds 8^3 finest cells
+
 struct RayWalk {
-  float go[3];     // grid position of the entry point (a multiple of 2^(depth-24))
-  float gd[3];     // grid-space direction (unit world direction * scale)
-  float inv[3];    // 1 / gd (inf when gd == 0)
-  float c[3];      // (exact entry - go) * inv: plane x lies at (x - go) * inv - c
+  float go[3];     // grid position of the entry point (a multiple of 2^(depth-24)), mirrored
+  float gd[3];     // size of the grid-space direction (unit world direction * scale)
+  float inv[3];    // 1 / gd (0 when gd == 0)
+  float c[3];      // (exact entry - go) * inv: plane x lies at (x - go) * inv - c (-inf when gd == 0)
+  int neg[3];      // -1 on a mirrored axis, else 0
+  uint32_t fwd;    // nibbles of a box code that hold the extents ahead of the ray
   float t_base;    // world distance of the entry point from the origin
   float t_cur;     // current distance past the entry point (hi part)
   float t_lo;      // its lo part (t_cur + t_lo: see the plane distances above)
   float t_far;     // exit distance of the root box past the entry point
-  int cell[3];
-  int steps, max_steps;
+  int cell[3];     // kMagicBits + the (mirrored) finest cell
+  int left;        // walk steps left before the step cap
   int restart;     // level at which the next descent may start (0 = root)
   uint32_t c_idx;  // brick-map cell of the last lookup (0xFFFFFFFF: none) ...
   uint32_t c_word; // ... and its word
@@ -173,6 +191,7 @@ __device__ __forceinline__ void walk_start(const DevTree &tr, const float p[3], 
   const int N = 1 << tr.depth;
   const float q = ldexpf(1.f, tr.depth - 24), iq = ldexpf(1.f, 24 - tr.depth);
   float tf = INFINITY;
+  uint32_t fwd = 0u;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     // grid coordinate gh + gl = (p + pl - bmin) * scale, then split at q
@@ -184,24 +203,30 @@ __device__ __forceinline__ void walk_start(const DevTree &tr, const float p[3], 
     if (gh >= (float)N) { gh = (float)N; gl = fminf(gl, 0.f); }
     const float go = rintf(gh * iq) * q;  // x - go is exact for integer x in [0, N]
     const float lo = (gh - go) + gl;
-    w.go[a] = go;
-    w.gd[a] = dn[a] * tr.scale[a];
-    w.inv[a] = w.gd[a] != 0.f ? 1.f / w.gd[a] : INFINITY;
-    w.c[a] = w.gd[a] != 0.f ? lo * w.inv[a] : 0.f;
+    const float gd = dn[a] * tr.scale[a];
+    const float inv = gd != 0.f ? 1.f / gd : 0.f;
     // the cell the ray occupies just after the exact entry point
-    int cell = cell_of(go, w.gd[a], N);
+    int cell = cell_of(go, gd, N);
     if (go == floorf(go) && lo != 0.f) cell = (lo < 0.f ? (int)go - 1 : (int)go);
-    w.cell[a] = min(max(cell, 0), N - 1);
-    if (w.gd[a] != 0.f) tf = fminf(tf, ((w.gd[a] > 0.f ? (float)N : 0.f) - go) * w.inv[a] - w.c[a]);
+    cell = min(max(cell, 0), N - 1);
+    const int neg = gd < 0.f ? -1 : 0;
+    w.go[a] = neg ? -go : go;
+    w.gd[a] = fabsf(gd);
+    w.inv[a] = fabsf(inv);
+    w.c[a] = gd != 0.f ? lo * inv : -INFINITY;
+    w.neg[a] = neg;
+    w.cell[a] = kMagicBits + (cell ^ neg);
+    fwd |= (neg ? 0x0Fu : 0xF0u) << (8 * a);
+    if (gd != 0.f) tf = fminf(tf, ((gd > 0.f ? (float)N : 0.f) - go) * inv - w.c[a]);
   }
+  w.fwd = fwd;
   w.t_cur = 0.f;
   w.t_lo = 0.f;
   w.t_far = tf;
   w.restart = 0;
   w.c_idx = 0xFFFFFFFFu;
   w.c_word = 0u;
-  w.steps = 0;
-  w.max_steps = tr.step_cap > 0 ? tr.step_cap : 3 * N + 8;
+  w.left = tr.step_cap > 0 ? tr.step_cap : 3 * N + 8;
   w.alive = tf > 0.f;
 }
 
@@ -269,11 +294,9 @@ struct PathRef {
 
 // Descends to the tree cell holding `cell`, from the root or (kPath) from the
 // ancestor at level `start` recorded by the previous descent.  Returns the
-// child entry found (kEmpty or kLeafBit|leaf) and its level.  The first
-// smem_nodes rows of the child table may be read from shared memory.
-template <bool kSmem, bool kPath>
-__device__ __forceinline__ uint32_t descend(const DevTree &tr, const uint32_t *s_child, PathRef pr, const int cell[3],
-                                            int start, int &level) {
+// child entry found (kEmpty or kLeafBit|leaf) and its level.
+template <bool kPath>
+__device__ __forceinline__ uint32_t descend(const DevTree &tr, PathRef pr, const int cell[3], int start, int &level) {
   const int D = tr.depth;
   uint32_t node = 0;
   int L = 0;
@@ -302,11 +325,7 @@ __device__ __forceinline__ uint32_t descend(const DevTree &tr, const uint32_t *s
     }
     const int bit = D - 1 - L;
     const int slot = (((cell[0] >> bit) & 1) << 2) | (((cell[1] >> bit) & 1) << 1) | ((cell[2] >> bit) & 1);
-    uint32_t e;
-    if (kSmem && node < (uint32_t)tr.smem_nodes)
-      e = s_child[node * 8 + slot];
-    else
-      e = __ldg(tr.child + (size_t)node * 8 + slot);
+    const uint32_t e = __ldg(tr.child + (size_t)node * 8 + slot);
     if (e == kEmpty || (e & kLeafBit)) {
       level = L + 1;
       if (e != kEmpty && (e & ~kLeafBit) >= (uint32_t)tr.n_leaves) {
@@ -331,166 +350,128 @@ __device__ __forceinline__ uint32_t descend(const DevTree &tr, const uint32_t *s
 // t0 of the segment's start past the entry point and its chord dt) when that
 // cell is an occupied leaf crossed with a positive chord.  Clears w.alive when
 // the ray leaves the root box or reaches its step cap.
-template <bool kSmem, bool kPath = false>
-__device__ __forceinline__ bool walk_step(const DevTree &tr, const uint32_t *s_child, RayWalk &w, uint32_t &leaf,
-                                          float &t0, float &dt, PathRef pr = PathRef{nullptr, 0}) {
-  const int N = 1 << tr.depth;
-  if (++w.steps > w.max_steps) {
+template <bool kPath = false>
+__device__ __forceinline__ bool walk_step(const DevTree &tr, RayWalk &w, uint32_t &leaf, float &t0, float &dt,
+                                          PathRef pr = PathRef{nullptr, 0}) {
+  if (w.left-- <= 0) {
     raise_status(tr, kStatusSegCap);
     w.alive = false;
     return false;
   }
-  // the box [lo, hi) the ray crosses next: the tree cell holding the current
-  // finest cell, or with a brick map possibly a larger empty box
-  uint32_t e;
-  int lo[3], hi[3];
-  bool fine = false;  // the box is a single finest cell
+  // the box the ray crosses next: the aligned cube of side m + 1 around the
+  // current finest cell, ext's forward extents << sx further ahead
+  const int mask = (1 << tr.depth) - 1;
+  const int x[3] = {(w.cell[0] ^ w.neg[0]) & mask, (w.cell[1] ^ w.neg[1]) & mask, (w.cell[2] ^ w.neg[2]) & mask};
+  uint32_t e = kEmpty, ext = 0u;
+  int m, sx = 0;
   if (tr.coarse) {
-    const int cs = tr.depth - tr.brick_level, Lc = tr.brick_level;
-    const int cx = w.cell[0] >> cs, cy = w.cell[1] >> cs, cz = w.cell[2] >> cs;
-    const uint32_t ci = ((uint32_t)cx << (2 * Lc)) | ((uint32_t)cy << Lc) | (uint32_t)cz;
+    const int Lc = tr.brick_level;
+    const uint32_t ci = ((uint32_t)(x[0] >> kBrickShift) << (2 * Lc)) + ((uint32_t)(x[1] >> kBrickShift) << Lc) +
+                        (uint32_t)(x[2] >> kBrickShift);
     if (ci != w.c_idx) {
       w.c_idx = ci;
       w.c_word = __ldg(tr.coarse + ci);
     }
-    const uint32_t cw = w.c_word, kind = cw >> 28;
-    if (kind == kCoarseEmpty) {
-      // the empty box around this brick-map cell: extents below and above
-      // it per axis, 4 bits each in units of 2^s cells
-      const int s = (int)((cw >> 24) & 15u), Nc = 1 << Lc;
-      const int cc[3] = {cx, cy, cz};
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        const int below = (int)((cw >> (8 * a)) & 15u) << s, above = (int)((cw >> (8 * a + 4)) & 15u) << s;
-        lo[a] = max(cc[a] - below, 0) << cs;
-        hi[a] = min(cc[a] + above + 1, Nc) << cs;
-      }
-      e = kEmpty;
+    uint32_t v = w.c_word;
+    if ((v >> 28) == kCoarseEmpty) {
+      // the empty box around this brick-map cell: extents in units of 2^s cells
+      m = (1 << kBrickShift) - 1;
+      ext = v;
+      sx = kBrickShift + (int)((v >> 24) & 15u);
     } else {
-      int level;
-      uint32_t box = 0u;  // an empty box's code from the brick (0: none)
-      if (kind == 0) {
-        const uint32_t b = cw & 0x0FFFFFFFu;
-        if (b >= (uint32_t)tr.brick_count) {
+      if ((v >> 28) == 0u) {
+        if (v >= (uint32_t)tr.brick_count) {
           raise_status(tr, kStatusBadIndex);
           w.alive = false;
           return false;
         }
-        const int m = (1 << cs) - 1;
-        const uint32_t idx = (uint32_t)(((w.cell[0] & m) << (2 * cs)) | ((w.cell[1] & m) << cs) | (w.cell[2] & m));
-        const uint32_t v = __ldg(tr.bricks + ((size_t)b << (3 * cs)) + idx);
-        level = (int)(v >> 28);
-        const uint32_t id = v & kBrickEmpty;
-        e = id >= kBrickBoxBase ? kEmpty : (kLeafBit | id);
-        if (id >= kBrickBoxBase && id != kBrickEmpty) box = id;  // an empty box around the cell
-      } else {
-        level = (int)kind;
-        e = kLeafBit | (cw & 0x0FFFFFFFu);
+        v = __ldg(tr.bricks + ((size_t)v << (3 * kBrickShift)) +
+                  (uint32_t)(((x[0] & 7) << 6) | ((x[1] & 7) << 3) | (x[2] & 7)));
       }
-      if (e != kEmpty && (e & ~kLeafBit) >= (uint32_t)tr.n_leaves) {
-        raise_status(tr, kStatusBadIndex);
-        e = kEmpty;
-      }
-      if (box) {
-        // extents below and above the cell per axis, 4 bits each
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-          lo[a] = w.cell[a] - (int)((box >> (8 * a)) & 15u);
-          hi[a] = w.cell[a] + (int)((box >> (8 * a + 4)) & 15u) + 1;
+      m = (1 << (tr.depth - (int)(v >> 28))) - 1;
+      const uint32_t id = v & kBrickEmpty;
+      if (id < kBrickBoxBase) {
+        e = kLeafBit | id;
+        if (id >= (uint32_t)tr.n_leaves) {
+          raise_status(tr, kStatusBadIndex);
+          e = kEmpty;
         }
-        fine = (box & 0x00FFFFFFu) == 0u;
-      } else {
-        const int size = 1 << (tr.depth - level);
-        fine = size == 1;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-          lo[a] = w.cell[a] & -size;
-          hi[a] = lo[a] + size;
-        }
+      } else if (id != kBrickEmpty) {  // an empty box around the cell
+        m = 0;
+        ext = id;
       }
     }
   } else {
     int level;
-    e = descend<kSmem, kPath>(tr, s_child, pr, w.cell, w.restart, level);
-    const int size = 1 << (tr.depth - level);
-    fine = size == 1;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      lo[a] = w.cell[a] & -size;
-      hi[a] = lo[a] + size;
-    }
+    e = descend<kPath>(tr, pr, x, w.restart, level);
+    m = (1 << (tr.depth - level)) - 1;
   }
+  // forward extents, one per byte
+  ext &= w.fwd;
+  ext = (ext | (ext >> 4)) & 0x000F0F0Fu;
+  int F[3];
   float gap[3], tx[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    gap[a] = (float)(w.gd[a] > 0.f ? hi[a] : lo[a]) - w.go[a];  // exact
+    F[a] = (w.cell[a] | m) + 1 + (int)(((ext >> (8 * a)) & 0xFFu) << sx);
+    gap[a] = (__int_as_float(F[a]) - kMagic) - w.go[a];  // exact
     // the plane's distance gap * inv - c with one rounding, so that the exit
-    // axis is decided on distances accurate to an ulp
-    tx[a] = w.gd[a] != 0.f ? fmaf(gap[a], w.inv[a], -w.c[a]) : INFINITY;
+    // axis is decided on distances accurate to an ulp (inf when gd == 0)
+    tx[a] = fmaf(gap[a], w.inv[a], -w.c[a]);
   }
   // exit axis: first minimum (exact ties x < y < z); register-only selects
-  int ax = 0;
-  float t_exit = tx[0], g_ax = gap[0], i_ax = w.inv[0], c_ax = w.c[0];
-  if (tx[1] < t_exit) { ax = 1; t_exit = tx[1]; g_ax = gap[1]; i_ax = w.inv[1]; c_ax = w.c[1]; }
-  if (tx[2] < t_exit) { ax = 2; t_exit = tx[2]; g_ax = gap[2]; i_ax = w.inv[2]; c_ax = w.c[2]; }
+  const bool y_first = tx[1] < tx[0];
+  float t_exit = y_first ? tx[1] : tx[0];
+  const bool z_first = tx[2] < t_exit;
+  const float g_ax = z_first ? gap[2] : (y_first ? gap[1] : gap[0]);
+  const float i_ax = z_first ? w.inv[2] : (y_first ? w.inv[1] : w.inv[0]);
+  const float c_ax = z_first ? w.c[2] : (y_first ? w.c[1] : w.c[0]);
+  t_exit = z_first ? tx[2] : t_exit;
+  const bool exits[3] = {!z_first && !y_first, !z_first && y_first, z_first};
   // the exit plane lies at t_exit + x_lo: x_lo = (gap * inv - t_exit) - c
   // (the product exact inside the FMA)
   const float x_lo = fmaf(g_ax, i_ax, -t_exit) - c_ax;
   const float chord = (t_exit - w.t_cur) + (x_lo - w.t_lo);
-  bool found = false;
-  if (e != kEmpty && chord > 0.f) {
-    leaf = e & ~kLeafBit;
-    t0 = w.t_cur;
-    dt = chord;
-    found = true;
-  }
+  const bool found = e != kEmpty && chord > 0.f;
+  leaf = e & ~kLeafBit;
+  t0 = w.t_cur;
+  dt = chord;
   // step to the next cell
   if (t_exit >= w.t_far) {
     w.alive = false;
-  } else {
-    if (chord > 0.f) {
-      w.t_cur = t_exit;
-      w.t_lo = x_lo;
-    }
-    // on the other axes the neighbour of a finest cell across the exit face
-    // has the same coordinates; a larger box needs the exit point's cell.
-    // The ray's coordinates move one way only, so a cell behind the current
-    // one on such an axis is the exit point's rounding (at an edge the ray
-    // crosses, the exit plane of one axis and a cell boundary of another at
-    // one distance) and is not taken: otherwise two boxes meeting at that
-    // edge could hand the walk back and forth without progress.
-    if (!fine) {
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        if (b != ax) {
-          const float p = fmaf(w.t_cur, w.gd[b], w.go[b]);
-          const int c = min(max(cell_of(p, w.gd[b], N), lo[b]), hi[b] - 1);
-          w.cell[b] = w.gd[b] > 0.f ? max(c, w.cell[b]) : (w.gd[b] < 0.f ? min(c, w.cell[b]) : c);
-        }
-      }
-    }
-    const int lo_ax = ax == 0 ? lo[0] : (ax == 1 ? lo[1] : lo[2]);
-    const int hi_ax = ax == 0 ? hi[0] : (ax == 1 ? hi[1] : hi[2]);
-    const float gd_ax = ax == 0 ? w.gd[0] : (ax == 1 ? w.gd[1] : w.gd[2]);
-    const int nc = gd_ax > 0.f ? hi_ax : lo_ax - 1;
-    const bool inside = nc >= 0 && nc < N;
-#pragma unroll
-    for (int b = 0; b < 3; ++b)
-      if (b == ax) w.cell[b] = nc;
-    // deepest level whose cell holds both the old node and the new cell
-    if (kPath && inside && !tr.coarse) w.restart = tr.depth - 32 + __clz(nc ^ lo_ax);
-    if (!inside) w.alive = false;
+    return found;
   }
+  if (chord > 0.f) {
+    w.t_cur = t_exit;
+    w.t_lo = x_lo;
+  }
+  // On the exit axis the cell across the plane; on the others the exit
+  // point's cell, within the box and never behind the current one.  The ray's
+  // coordinates move one way only, so a cell behind is the exit point's
+  // rounding (at an edge the ray crosses, the exit plane of one axis and a
+  // cell boundary of another at one distance) and is not taken: otherwise two
+  // boxes meeting at that edge could hand the walk back and forth without
+  // progress.  (Across a finest cell this keeps the other coordinates.)
+  bool out = false;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const float p = fmaf(w.t_cur, w.gd[a], w.go[a]);
+    const int c = max(min(__float_as_int(__fadd_rd(p, kMagic)), F[a] - 1), w.cell[a]);
+    const int n = exits[a] ? F[a] : c;
+    // deepest level whose cell holds both the old node and the new cell
+    if (kPath && exits[a] && !tr.coarse) w.restart = tr.depth - 32 + __clz((n ^ w.cell[a]) & mask);
+    w.cell[a] = n;
+    out = out || (((n ^ w.neg[a]) >> tr.depth) & 1) != 0;  // cell N or -1
+  }
+  if (out) w.alive = false;
   return found;
 }
 
 // Advances to the next occupied-leaf segment (see walk_step); false when the
 // ray has left the root box (or hit its step cap).
-template <bool kSmem, bool kPath = false>
-__device__ __forceinline__ bool walk_next(const DevTree &tr, const uint32_t *s_child, RayWalk &w, uint32_t &leaf,
-                                          float &t0, float &dt, PathRef pr = PathRef{nullptr, 0}) {
+__device__ __forceinline__ bool walk_next(const DevTree &tr, RayWalk &w, uint32_t &leaf, float &t0, float &dt) {
   while (w.alive)
-    if (walk_step<kSmem, kPath>(tr, s_child, w, leaf, t0, dt, pr)) return true;
+    if (walk_step(tr, w, leaf, t0, dt)) return true;
   return false;
 }
 

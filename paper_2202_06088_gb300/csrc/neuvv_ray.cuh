@@ -18,8 +18,8 @@ struct RayResult {
 // that brings the transmittance below t_stop.  dn: unit direction in the
 // tree's frame (the view direction of the harmonics); u: frame coordinate;
 // t_base + dist_scale * t converts a walk distance t to the caller's frame.
-template <int KP, int DEG, typename E, bool kSmem>
-__device__ __forceinline__ void integrate_walk(const DevTree &tr, const uint32_t *s_child, RayWalk &w,
+template <int KP, int DEG, typename E>
+__device__ __forceinline__ void integrate_walk(const DevTree &tr, RayWalk &w,
                                                const float dn[3], float u, float t_stop, int act, float t_base,
                                                float dist_scale, RayResult &res) {
   RayConst<KP, DEG> rc;
@@ -28,7 +28,7 @@ __device__ __forceinline__ void integrate_walk(const DevTree &tr, const uint32_t
   float T = 1.f;
   uint32_t leaf;
   float t0, dt;
-  while (walk_next<kSmem>(tr, s_child, w, leaf, t0, dt)) {
+  while (walk_next(tr, w, leaf, t0, dt)) {
     LeafRecord<KP, DEG, E> rec;
     rec.load(tr, leaf);
     Sample<DEG> s;
@@ -58,14 +58,14 @@ __device__ __forceinline__ void clear(RayResult &res) {
 }
 
 // One ray given in the tree's own frame (render kernels).
-template <int KP, int DEG, typename E, bool kSmem>
-__device__ __forceinline__ void integrate_ray(const DevTree &tr, const uint32_t *s_child, const float o[3],
+template <int KP, int DEG, typename E>
+__device__ __forceinline__ void integrate_ray(const DevTree &tr, const float o[3],
                                               const float d[3], float u, float t_stop, int act, RayResult &res) {
   clear(res);
   RayWalk w;
   float dn[3];
   if (!walk_init(tr, o, d, w, dn)) return;
-  integrate_walk<KP, DEG, E, kSmem>(tr, s_child, w, dn, u, t_stop, act, w.t_base, 1.f, res);
+  integrate_walk<KP, DEG, E>(tr, w, dn, u, t_stop, act, w.t_base, 1.f, res);
 }
 
 __device__ __forceinline__ float depth_of(const RayResult &r) { return r.A >= 1e-4f ? r.dnum / r.A : INFINITY; }

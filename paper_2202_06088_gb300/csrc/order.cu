@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(256) ray_key_kernel(const __grid_constant__ De
   RayWalk w;
   uint32_t leaf, key = kMissKey;
   float t0, dt;
-  if (walk_init(tr, o, d, w, dn) && walk_next<false>(tr, nullptr, w, leaf, t0, dt))
+  if (walk_init(tr, o, d, w, dn) && walk_next(tr, w, leaf, t0, dt))
     key = (direction_bucket(dn) << 18) | ((leaf >> shift) & 0x3FFFFu);
   keys[i] = key;
   perm[i] = (uint32_t)i;

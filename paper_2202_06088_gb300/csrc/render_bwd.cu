@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(256) render_bwd_plain_kernel(const __grid_cons
   sh_real<DEG>(dn, rc.Y);
   uint32_t leaf;
   float t0, dt;
-  while (st.count < st.target && walk_next<false>(a.tr, nullptr, w, leaf, t0, dt)) {
+  while (st.count < st.target && walk_next(a.tr, w, leaf, t0, dt)) {
     ++st.count;
     adjoint_sample<KP, DEG, E>(a, RegRows<KP>{rc.a, rc.b}, rc.Y, leaf, dt, st);
   }
@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(256) packet_key_kernel(const __grid_constant__
     RayWalk w;
     uint32_t leaf;
     float t0, dt;
-    if (walk_init(tr, o, d, w, dn) && walk_next<false>(tr, nullptr, w, leaf, t0, dt)) key = leaf;
+    if (walk_init(tr, o, d, w, dn) && walk_next(tr, w, leaf, t0, dt)) key = leaf;
   }
   l.key[p] = key;
 }
@@ -443,7 +443,7 @@ __device__ __noinline__ void adjoint_walk_packet(const BwdArgs &a, long long i, 
     if (walking && qn < queue) {
       uint32_t leaf;
       float t0, dt;
-      if (walk_step<false, true>(tr, nullptr, w, leaf, t0, dt, pr)) {
+      if (walk_step<true>(tr, w, leaf, t0, dt, pr)) {
         const int slot = (qh + qn) & qmask;
         q_leaf[slot * B] = leaf;
         q_dt[slot * B] = dt;

@@ -18,7 +18,7 @@ __global__ void __launch_bounds__(256) render_plain_kernel(const __grid_constant
   float o[3], d[3], t;
   load_ray(a.rays, i, o, d, t);
   RayResult r;
-  integrate_ray<KP, DEG, E, false>(a.tr, nullptr, o, d, t * (float)(a.tr.T - 1), a.t_stop, a.act, r);
+  integrate_ray<KP, DEG, E>(a.tr, o, d, t * (float)(a.tr.T - 1), a.t_stop, a.act, r);
   a.out.rgb[3 * i + 0] = r.C[0];
   a.out.rgb[3 * i + 1] = r.C[1];
   a.out.rgb[3 * i + 2] = r.C[2];
@@ -98,7 +98,7 @@ __device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pos, 
     if (walking && qn < queue) {
       uint32_t leaf;
       float t0, dt;
-      if (walk_step<false, true>(tr, nullptr, w, leaf, t0, dt, pr)) {
+      if (walk_step<true>(tr, w, leaf, t0, dt, pr)) {
         const int slot = (qh + qn) & qmask;
         q_leaf[slot * B] = leaf;
         q_t0[slot * B] = t0;
@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(256) trace_kernel(const __grid_constant__ Trac
   if (walk_init(a.tr, o, d, w, dn)) {
     uint32_t leaf;
     float t0, dt;
-    while (walk_next<false>(a.tr, nullptr, w, leaf, t0, dt)) {
+    while (walk_next(a.tr, w, leaf, t0, dt)) {
       if (c < a.max_out) {
         a.leaf[i * a.max_out + c] = (int)leaf;
         a.t0[i * a.max_out + c] = w.t_base + t0;
@@ -598,9 +598,9 @@ __global__ void __launch_bounds__(256) pick_kernel(const __grid_constant__ FwdAr
     float optical = 0.f;
     uint32_t leaf;
     float t0, dt;
-    while (walk_next<false>(a.tr, nullptr, w, leaf, t0, dt)) {
+    while (walk_next(a.tr, w, leaf, t0, dt)) {
       LeafRecord<KP, DEG, E> rec;
-      rec.load(a.tr, leaf);
+      rec.load_sigma(a.tr, leaf);
       optical = fmaf(fmaxf(pre_sigma_of<KP>(rows, rec), 0.f), dt, optical);
       if (-expm1f(-optical) >= threshold) {
         picked = (int)leaf;
