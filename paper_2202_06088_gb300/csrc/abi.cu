@@ -93,7 +93,7 @@ struct neuvv_tree {
   float hh_norm[16];
   int num_sms = 0;
   LaunchCfg plain{128, 1, 1, 0, 0, 0};
-  LaunchCfg packet{64, 8, 16, 0, 1, 0};
+  LaunchCfg packet{64, 8, 32, 0, 1, 0};
   LaunchCfg compose{128, 1, 1, 0, 1, 0};
   int step_cap = 0;             // walk steps per ray (0: 3 * 2^depth + 8)
   int wait_polls = 1 << 22;     // polls of a bounded device wait
@@ -158,7 +158,7 @@ DevRays dev_rays(const neuvv_rays *r, float t) {
 
 // Device view of a caller's segment log buffer (layout private to the
 // library): 64-byte header, heads, key and order [n_packets], perm [n_rays],
-// the sort bins, next [n_chunks], then leaf and chord planes of n_chunks x
+// the sort bins, next [n_chunks], then leaf, chord and lane planes of n_chunks x
 // kLogRounds x 32 entries.  n_chunks = 0 when the buffer is absent or too
 // small for one chunk.  *chunk_bytes (nullable) receives the bytes from the
 // start of next[] to the end of the buffer (scratch for a ray order before
@@ -175,7 +175,7 @@ SampleLog log_view(void *base, int64_t bytes, int64_t n_rays, int64_t *chunk_byt
   const int64_t pk_bytes = (4 * n_packets + 15) / 16 * 16;
   const int64_t perm_bytes = (4 * n_rays + 15) / 16 * 16;
   const int64_t fixed = 64 + 3 * pk_bytes + perm_bytes + 4 * kSortBins;
-  const int64_t per_chunk = 4 + (int64_t)kLogRounds * 32 * 8;
+  const int64_t per_chunk = 4 + (int64_t)kLogRounds * 32 * 9;
   const int64_t avail = bytes - fixed - 16;
   if (avail < per_chunk) return l;
   int64_t nc = avail / per_chunk;
@@ -189,6 +189,7 @@ SampleLog log_view(void *base, int64_t bytes, int64_t n_rays, int64_t *chunk_byt
   const int64_t leaf_off = (fixed + 4 * nc + 15) / 16 * 16;
   l.leaf = reinterpret_cast<uint32_t *>(p + leaf_off);
   l.dt = reinterpret_cast<float *>(p + leaf_off + nc * kLogRounds * 32 * 4);
+  l.lane = reinterpret_cast<uint8_t *>(l.dt + nc * kLogRounds * 32);
   l.n_chunks = (uint32_t)nc;
   if (chunk_bytes) *chunk_bytes = bytes - fixed;
   return l;
@@ -1535,7 +1536,7 @@ neuvv_status neuvv_autotune(neuvv_tree *t, const neuvv_rays *sample, float time,
   float best_t = 1e30f;
   std::vector<neuvv_tune_entry> table;
   struct Cand { int block, queue, ready; };
-  const Cand cands[] = {{64, 8, 16}, {64, 1, 1}, {64, 4, 8}, {128, 8, 16}, {128, 1, 1}, {32, 8, 16}, {64, 16, 16}};
+  const Cand cands[] = {{64, 8, 32}, {64, 8, 24}, {64, 8, 16}, {128, 8, 32}, {32, 8, 32}};
   for (int order = NEUVV_ORDER_AS_GIVEN; order <= NEUVV_ORDER_BY_RAY && s == NEUVV_OK; ++order)
     for (const Cand &c : cands) {
       t->packet = saved;

@@ -11,8 +11,8 @@ enum DType { kF32 = 0, kBF16 = 1, kFP8 = 2 };
 
 struct LaunchCfg {
   int block;          // threads per block
-  int queue;          // packet kernels: per-lane queue of found leaf segments (power of 2, <= kMaxQueue)
-  int ready;          // packet kernels: lanes with a queued segment that trigger a shading round
+  int queue;          // packet kernels: kept as set by the caller (segments wait in one ring per packet)
+  int ready;          // packet kernels: waiting segments that start a shading round
   int grid;           // compose: persistent blocks (0 = as many as fit, from the occupancy API)
   int dynamic_queue;  // compose and the packet forward: 1 = persistent warps pull 32-ray
                       // packets from a counter, 0 = one packet per warp of the grid
@@ -23,8 +23,9 @@ struct LaunchCfg {
 };
 
 // Segment log of the packet forward (device view of neuvv_out.log).  Chunks
-// of kLogRounds shading rounds x 32 lanes hold (leaf, chord) per lane, kEmpty
-// for a lane that shaded nothing in that round; a packet's chunks are linked
+// of kLogRounds shading rounds x 32 slots hold (leaf, chord, lane of the
+// ray) per composited segment, a ray's segments in order, leaf = kEmpty in a
+// slot without one; a packet's chunks are linked
 // from heads[packet] through next[].  heads[packet] = kNoLog: not logged
 // (replay by walking).  Header: chunk counter (u64), then n_chunks, rounds,
 // n_rays (i64), a valid word and a permuted word, all written by the forward
@@ -43,6 +44,7 @@ struct SampleLog {
   uint32_t *next;     // [n_chunks]
   uint32_t *leaf;     // [n_chunks][kLogRounds][32]
   float *dt;          // [n_chunks][kLogRounds][32]
+  uint8_t *lane;      // [n_chunks][kLogRounds][32] the packet's lane whose ray a slot belongs to
   uint32_t n_chunks;  // 0: no log
 };
 constexpr uint32_t kNoKey = 0xFFFFFFFFu;
@@ -240,14 +242,18 @@ cudaError_t launch_mse(const float *rgb, const float *target, long long n, float
 cudaError_t launch_grad_loss(const float *rgb, const float *target, const int *map, int width, int height,
                              long long n_views, long long n_rays, float lam, float *grad, float *loss, cudaStream_t s);
 
-// Dynamic shared memory of the packet kernels: per thread the basis rows
-// (2 K_pad floats), the descent path (kPathWords levels; none for a tree with
-// a brick map, whose walk never descends the child table) and the segment
-// queue (queue x {leaf, t0, t1}).
+// Shared memory of a packet kernel, per warp: a ring of the segments that wait
+// for shading (room for a batch of 32 and one step's finds), and per thread
+// the entries a ray owns in the current batch, the adjoint's per-entry result
+// (two words), the ray's unit direction, its basis rows (2 K_pad floats) and
+// the descent path (kPathWords levels; none for a tree with a brick map,
+// whose walk never descends the child table).
+constexpr int kRing = 64;
 constexpr int kPathWords = 16;
 __host__ __device__ inline int path_words(const DevTree &tr) { return tr.path_words; }
-inline size_t smem_bytes(int block, int KP, int queue, const DevTree &tr) {
-  return (size_t)block * (2 * KP + path_words(tr) + 3 * queue) * sizeof(float);
+constexpr int kPacketWords = 4 * kRing / 32 + 1 + 2 + 3;
+inline size_t smem_bytes(int block, int KP, const DevTree &tr) {
+  return (size_t)block * (kPacketWords + 2 * KP + path_words(tr)) * sizeof(float);
 }
 constexpr int kMaxQueue = 32;
 // Packet kernels are latency bound: two 256-thread blocks per SM (128

@@ -2,7 +2,7 @@
 // compose kernels (Sec. 4.3 "Rendering"; Eq. volume-rendering).
 #pragma once
 
-#include "neuvv_device.cuh"
+#include "neuvv_kernels.h"
 
 namespace neuvv {
 
@@ -67,6 +67,61 @@ __device__ __forceinline__ void integrate_ray(const DevTree &tr, const float o[3
   if (!walk_init(tr, o, d, w, dn)) return;
   integrate_walk<KP, DEG, E>(tr, w, dn, u, t_stop, act, w.t_base, 1.f, res);
 }
+
+// ---------------------------------------------------------------------------
+// Packets: the 32 rays of a warp walk independently, and the segments they
+// find wait in one ring of the warp.  A batch of up to 32 waiting segments is
+// evaluated one per lane whichever rays they belong to -- a sample is some
+// six hundred instructions, and packets of uneven or incoherent rays would
+// run them with few lanes active if each lane shaded its own ray's segments
+// only -- and each ray then composites its own entries of the batch in order.
+// ---------------------------------------------------------------------------
+constexpr unsigned kFull = 0xFFFFFFFFu;
+
+// Pointers into a packet kernel's dynamic shared memory (kPacketWords).
+template <int KP>
+struct PacketShared {
+  uint4 *ring;      // [kRing] leaf, chord, distance of its middle, lane of the ray
+  unsigned *own;    // [32] entries of the batch that belong to each lane's ray
+  float2 *res;      // [32] per entry of the batch (the adjoint)
+  float *dn, *rows; // unit direction and basis rows of lane 0's ray; next lane +1, next value +stride
+  uint32_t *path;   // this thread's descent path, next level +stride
+  int stride;
+  __device__ __forceinline__ explicit PacketShared(uint32_t *smem) {
+    const int B = blockDim.x, w0 = threadIdx.x & ~31;
+    ring = reinterpret_cast<uint4 *>(smem) + 2 * w0;
+    uint32_t *p = smem + 4 * kRing / 32 * B;
+    own = p + w0;
+    res = reinterpret_cast<float2 *>(p + B) + w0;
+    dn = reinterpret_cast<float *>(p + 3 * B) + w0;
+    rows = reinterpret_cast<float *>(p + 6 * B) + w0;
+    path = p + (6 + 2 * KP) * B + threadIdx.x;
+    stride = B;
+  }
+  // This thread's ray, for the batch evaluation (any lane may shade it).
+  __device__ __forceinline__ void put_ray(const DevTree &tr, const float d[3], float u, bool with_rows) const {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) dn[k * stride + lane] = d[k];
+    if (with_rows) rows_to_smem<KP>(tr, u, rows + lane, stride);
+  }
+  __device__ __forceinline__ void get_dir(int lane, float d[3]) const {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) d[k] = dn[k * stride + lane];
+  }
+  __device__ __forceinline__ SmemRows<KP> rows_of(int lane) const { return SmemRows<KP>{rows + lane, stride}; }
+  // Entries of the batch that belong to this lane's ray, as a mask (entry j
+  // of `owner` in lane j when has).
+  __device__ __forceinline__ unsigned entries_of_lane(bool has, int owner) const {
+    const int lane = threadIdx.x & 31;
+    const unsigned grp = __match_any_sync(kFull, has ? owner : 32 + lane);
+    own[lane] = 0u;
+    __syncwarp();
+    if (has && lane == __ffs(grp) - 1) own[owner] = grp;
+    __syncwarp();
+    return own[lane];
+  }
+};
 
 __device__ __forceinline__ float depth_of(const RayResult &r) { return r.A >= 1e-4f ? r.dnum / r.A : INFINITY; }
 

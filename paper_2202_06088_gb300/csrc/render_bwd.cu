@@ -37,39 +37,64 @@ struct AdjState {
   int count, target;
 };
 
-// Gradient factors of one sample: with them, dL/dw_sigma = dpre_s a(u),
-// dL/dw_gamma = dpre_g b(u) and dL/dw_HH[ch][n,l,m] = R_nl(gamma) F[ch][l,m]
-// with F[ch][l,m] = dz[ch] Y_lm.  Advances the ray's replay state; false when
-// the sample has zero density (no path from it to the loss).
+// A sample's share of the adjoint that only its own record and chord decide.
+template <int DEG>
+struct SampleTerms {
+  Sample<DEG> s;
+  float ex, al;  // exp(-sigma delta), 1 - exp(-sigma delta); 1 and 0 for zero density
+};
+
+// Evaluates one sample; false when it has zero density (no path from it to
+// the loss).
 template <int KP, int DEG, typename E, typename Rows>
-__device__ __forceinline__ bool sample_factors(const BwdArgs &a, const Rows &rows, const float *Y, uint32_t leaf,
-                                               float dt, AdjState &st, Sample<DEG> &s, float dz[3], float &dpre_s,
-                                               float &dpre_g) {
-  const DevTree &tr = a.tr;
+__device__ __forceinline__ bool sample_terms(const BwdArgs &a, const Rows &rows, const float *Y, uint32_t leaf, float dt,
+                                             SampleTerms<DEG> &m) {
   LeafRecord<KP, DEG, E> rec;
-  rec.load(tr, leaf);
-  eval_sample<KP, DEG, E, Rows, true>(tr, rows, Y, rec, a.act, s);
-  if (!(s.sigma > 0.f)) return false;
-  const float sd = s.sigma * dt;
-  const float e = __expf(-sd);
-  const float wgt = st.T * alpha_of(sd);
-  const float Tn = st.T * e;
-  float dsig = st.gA * st.T_final;
+  rec.load(a.tr, leaf);
+  eval_sample<KP, DEG, E, Rows, true>(a.tr, rows, Y, rec, a.act, m.s);
+  m.ex = 1.f;
+  m.al = 0.f;
+  if (!(m.s.sigma > 0.f)) {
+    m.s.c[0] = m.s.c[1] = m.s.c[2] = 0.f;
+    return false;
+  }
+  const float sd = m.s.sigma * dt;
+  m.ex = __expf(-sd);
+  m.al = alpha_of(sd);
+  return true;
+}
+
+// Advances a ray's replay state over one sample (its terms al, ex and colour
+// c): the sample's weight and dL/dsigma per unit chord.
+__device__ __forceinline__ void replay_sample(AdjState &st, float al, float ex, const float c[3], float &wgt,
+                                              float &dsig) {
+  wgt = st.T * al;
+  const float Tn = st.T * ex;
+  dsig = st.gA * st.T_final;
 #pragma unroll
   for (int ch = 0; ch < 3; ++ch) {
-    st.acc[ch] = fmaf(wgt, s.c[ch], st.acc[ch]);
+    st.acc[ch] = fmaf(wgt, c[ch], st.acc[ch]);
     const float S_after = st.C[ch] - st.acc[ch];
-    dsig = fmaf(st.g[ch], Tn * s.c[ch] - S_after, dsig);
-    const float dc = wgt * st.g[ch];
+    dsig = fmaf(st.g[ch], Tn * c[ch] - S_after, dsig);
+  }
+  st.T = Tn;
+}
+
+// Gradient factors of one sample: with them, dL/dw_sigma = dpre_s a(u),
+// dL/dw_gamma = dpre_g b(u) and dL/dw_HH[ch][n,l,m] = R_nl(gamma) F[ch][l,m]
+// with F[ch][l,m] = dz[ch] Y_lm.
+template <int DEG>
+__device__ __forceinline__ void factors_of(const BwdArgs &a, const Sample<DEG> &s, const float g[3], float wgt,
+                                           float dsig, float dt, float dz[3], float &dpre_s, float &dpre_g) {
+#pragma unroll
+  for (int ch = 0; ch < 3; ++ch) {
+    const float dc = wgt * g[ch];
     dz[ch] = a.act == 0 ? dc * s.c[ch] * (1.f - s.c[ch]) : dc;
   }
-  dsig *= dt;
-  st.T = Tn;
   // dL/dgamma = sum_ch dz[ch] d z_ch / dgamma
   const float dgam = dz[0] * s.u[0] + dz[1] * s.u[1] + dz[2] * s.u[2];
   dpre_g = dgam * kPi * s.s_gamma * (1.f - s.s_gamma);
-  dpre_s = s.pre_sigma > 0.f ? dsig : 0.f;
-  return true;
+  dpre_s = s.pre_sigma > 0.f ? dsig * dt : 0.f;
 }
 
 // Scatters a leaf's gradient from its factors into its FP32 record with
@@ -119,61 +144,17 @@ template <int KP, int DEG, typename E, typename Rows>
 __device__ __forceinline__ void adjoint_sample(const BwdArgs &a, const Rows &rows, const float *Y, uint32_t leaf,
                                                float dt, AdjState &st) {
   constexpr int NY = (DEG + 1) * (DEG + 1);
-  Sample<DEG> s;
-  float dz[3], dpre_s, dpre_g;
-  if (!sample_factors<KP, DEG, E, Rows>(a, rows, Y, leaf, dt, st, s, dz, dpre_s, dpre_g)) return;
+  SampleTerms<DEG> m;
+  if (!sample_terms<KP, DEG, E>(a, rows, Y, leaf, dt, m)) return;
+  float wgt, dsig, dz[3], dpre_s, dpre_g;
+  replay_sample(st, m.al, m.ex, m.s.c, wgt, dsig);
+  factors_of<DEG>(a, m.s, st.g, wgt, dsig, dt, dz, dpre_s, dpre_g);
   float F[3 * NY];
 #pragma unroll
   for (int ch = 0; ch < 3; ++ch)
 #pragma unroll
     for (int k = 0; k < NY; ++k) F[ch * NY + k] = dz[ch] * Y[k];
-  scatter_gradient<KP, DEG, Rows>(a, rows, leaf, s.R, F, dpre_s, dpre_g);
-}
-
-// Adjoint of one shading round of a packet, called by every present lane;
-// `has` marks the lanes that hold a sample.  Warp-aggregated scatter: lanes
-// whose samples share a leaf and a time (hence the basis rows a(u), b(u) and
-// the hyper-angle, so the radial factors R_nl) add their factors dpre_s,
-// dpre_g and F[ch][l,m] with shuffles, and the lowest lane of each such group
-// scatters the group's gradient: one set of vector atomics per distinct
-// (leaf, time) in the round instead of one per sample.
-template <int KP, int DEG, typename E, typename Rows>
-__device__ __forceinline__ void adjoint_round(const BwdArgs &a, const Rows &rows, const float *Y, uint32_t leaf,
-                                              float dt, float t, bool has, unsigned present, AdjState &st) {
-  constexpr int NY = (DEG + 1) * (DEG + 1);
-  const int lane = threadIdx.x & 31;
-  Sample<DEG> s;
-  float dz[3] = {0.f, 0.f, 0.f}, dpre_s = 0.f, dpre_g = 0.f;
-  const bool contrib = has && sample_factors<KP, DEG, E, Rows>(a, rows, Y, leaf, dt, st, s, dz, dpre_s, dpre_g);
-  // lanes without a contribution get keys of their own (leaf ids are < 2^31)
-  const unsigned long long key =
-      contrib ? (((unsigned long long)leaf << 32) | __float_as_uint(t)) : (~0ull - (unsigned long long)lane);
-  const unsigned grp = __match_any_sync(present, key);
-  const bool leader = contrib && lane == __ffs(grp) - 1;
-  float F[3 * NY];
-#pragma unroll
-  for (int ch = 0; ch < 3; ++ch)
-#pragma unroll
-    for (int k = 0; k < NY; ++k) F[ch * NY + k] = dz[ch] * Y[k];
-  const int gmax = (int)__reduce_max_sync(present, contrib ? (unsigned)__popc(grp) : 1u);
-  unsigned rest = leader ? (grp & (grp - 1u)) : 0u;  // the leader's other members
-  for (int it = 1; it < gmax; ++it) {
-    const int src = rest ? __ffs(rest) - 1 : lane;
-    rest &= rest - 1u;
-    const bool add = src != lane;
-    const float xs = __shfl_sync(present, dpre_s, src);
-    const float xg = __shfl_sync(present, dpre_g, src);
-    if (add) {
-      dpre_s += xs;
-      dpre_g += xg;
-    }
-#pragma unroll
-    for (int k = 0; k < 3 * NY; ++k) {
-      const float x = __shfl_sync(present, F[k], src);
-      if (add) F[k] += x;
-    }
-  }
-  if (leader) scatter_gradient<KP, DEG, Rows>(a, rows, leaf, s.R, F, dpre_s, dpre_g);
+  scatter_gradient<KP, DEG, Rows>(a, rows, leaf, m.s.R, F, dpre_s, dpre_g);
 }
 
 // Octahedral code of a unit direction (the direction divided by its L1 norm,
@@ -205,44 +186,128 @@ __device__ __forceinline__ void oct_decode(float e0, float e1, float d[3]) {
   d[2] = z * il;
 }
 
-// Adjoint of one shading round for the leaf-major reduction, called by every
-// present lane; `has` marks the lanes that hold a sample.  Each sample takes
-// the next position of its leaf's run (lanes of the round that share a leaf
-// take consecutive positions with one atomic), reserved before the sample is
-// evaluated so that the atomic's round trip overlaps the evaluation, and
-// leaves its gradient factors (dpre_s, dpre_g, dz), its ray's frame
-// coordinate u and the octahedral code of its unit direction there.  A
-// sample of zero density leaves a record marked kNoFactor.  No gradient
-// atomics; the per-leaf sums are formed by leaf_reduce_kernel.
-template <int KP, int DEG, typename E, typename Rows>
-__device__ __forceinline__ void adjoint_round_gather(const BwdArgs &a, const Rows &rows, const float *Y, uint32_t leaf,
-                                                     float dt, float u, const float dn[3], bool has, unsigned present,
-                                                     AdjState &st) {
+// Adjoint of one batch of a packet's samples, called by the whole warp: lane j
+// holds entry j (leaf, dt, the lane `owner` of its ray; has: a sample, valid:
+// one whose leaf exists), a ray's entries in order.  Each entry is evaluated by its lane; each ray then
+// runs its replay state over its own entries (at most target - count of them)
+// and leaves every entry's weight and dL/dsigma in shared memory, from which
+// the entry's lane forms the gradient factors.
+//
+// With kGather (leaf-major reduction) each sample takes the next position of
+// its leaf's run (lanes of the batch that share a leaf take consecutive
+// positions with one atomic), reserved before the sample is evaluated so that
+// the atomic's round trip overlaps the evaluation, and leaves its factors
+// (dpre_s, dpre_g, dz), its ray's frame coordinate u and the octahedral code
+// of its unit direction there; a sample of zero density leaves a record marked
+// kNoFactor.  No gradient atomics; the per-leaf sums are formed by
+// leaf_reduce_kernel.
+//
+// Otherwise a warp-aggregated scatter: lanes whose samples share a leaf and a
+// time (hence the basis rows a(u), b(u) and the hyper-angle, so the radial
+// factors R_nl) add their factors dpre_s, dpre_g and F[ch][l,m] with shuffles,
+// and the lowest lane of each such group scatters the group's gradient: one
+// set of vector atomics per distinct (leaf, time) in the batch instead of one
+// per sample.
+template <int KP, int DEG, typename E, bool kGather>
+__device__ __forceinline__ void adjoint_batch(const BwdArgs &a, const PacketShared<KP> &sh, uint32_t leaf, float dt,
+                                              int owner, bool has, bool valid, float t,
+                                              AdjState &st) {
+  constexpr int NY = (DEG + 1) * (DEG + 1);
   const int lane = threadIdx.x & 31;
   uint32_t base = 0u;
-  {
-    const unsigned grp = __match_any_sync(present, has ? leaf : kEmpty);
-    if (has && lane == __ffs(grp) - 1) base = atomicAdd(a.gws.cur + leaf, (uint32_t)__popc(grp));
+  if (kGather) {
+    const unsigned grp = __match_any_sync(kFull, valid ? leaf : kEmpty);
+    if (valid && lane == __ffs(grp) - 1) base = atomicAdd(a.gws.cur + leaf, (uint32_t)__popc(grp));
   }
-  Sample<DEG> s;
+  float dn[3], Y[NY];
+  sh.get_dir(owner, dn);
+  sh_real<DEG>(dn, Y);
+  const SmemRows<KP> rows = sh.rows_of(owner);
+  SampleTerms<DEG> m;
+  m.al = 0.f;
+  m.ex = 1.f;
+  m.s.c[0] = m.s.c[1] = m.s.c[2] = 0.f;
+  const bool dense = valid && sample_terms<KP, DEG, E>(a, rows, Y, leaf, dt, m);
+  unsigned mine = sh.entries_of_lane(has, owner), kept = 0u;
+  while (__any_sync(kFull, mine != 0u)) {
+    const int j = mine ? __ffs(mine) - 1 : lane;
+    const float al = __shfl_sync(kFull, m.al, j), ex = __shfl_sync(kFull, m.ex, j);
+    float c[3];
+#pragma unroll
+    for (int ch = 0; ch < 3; ++ch) c[ch] = __shfl_sync(kFull, m.s.c[ch], j);
+    if (mine) {
+      mine &= mine - 1u;
+      if (st.count < st.target) {
+        ++st.count;
+        kept |= 1u << j;
+        float wgt, dsig;
+        replay_sample(st, al, ex, c, wgt, dsig);
+        sh.res[j] = make_float2(wgt, dsig);
+      }
+    }
+  }
+  kept = __reduce_or_sync(kFull, kept);
+  const bool contrib = dense && ((kept >> lane) & 1u);
+  float g[3];
+#pragma unroll
+  for (int ch = 0; ch < 3; ++ch) g[ch] = __shfl_sync(kFull, st.g[ch], owner);
+  const float to = __shfl_sync(kFull, t, owner);  // the entry's time
+  __syncwarp();
   float dz[3] = {0.f, 0.f, 0.f}, dpre_s = 0.f, dpre_g = 0.f;
-  const bool contrib = has && sample_factors<KP, DEG, E, Rows>(a, rows, Y, leaf, dt, st, s, dz, dpre_s, dpre_g);
-  // the group again (recomputed rather than held through the evaluation)
-  const unsigned grp = __match_any_sync(present, has ? leaf : kEmpty);
-  base = __shfl_sync(present, base, __ffs(grp) - 1);
-  if (!has) return;
-  const uint32_t p = base + (uint32_t)__popc(grp & ((1u << lane) - 1u));
-  // the count over the log bounds every run; this keeps a write inside the
-  // workspace even if the log changed between the count and the replay
-  if (p >= a.gws.cap_chunks * (uint32_t)(kLogRounds * 32)) {
-    raise_status(a.tr, kStatusBadIndex);
-    return;
+  if (contrib) {
+    const float2 r = sh.res[lane];
+    factors_of<DEG>(a, m.s, g, r.x, r.y, dt, dz, dpre_s, dpre_g);
   }
-  float e0 = kNoFactor, e1 = 0.f;
-  if (contrib) oct_encode(dn, e0, e1);
-  float4 *f = a.gws.fac + 2 * (size_t)p;
-  __stcs(f, make_float4(dpre_s, dpre_g, dz[0], dz[1]));
-  __stcs(f + 1, make_float4(dz[2], u, e0, e1));
+  if constexpr (kGather) {
+    // the group again (recomputed rather than held through the evaluation)
+    const unsigned grp = __match_any_sync(kFull, valid ? leaf : kEmpty);
+    base = __shfl_sync(kFull, base, __ffs(grp) - 1);
+    if (valid) {
+      const uint32_t p = base + (uint32_t)__popc(grp & ((1u << lane) - 1u));
+      // the count over the log bounds every run; this keeps a write inside the
+      // workspace even if the log changed between the count and the replay
+      if (p >= a.gws.cap_chunks * (uint32_t)(kLogRounds * 32)) {
+        raise_status(a.tr, kStatusBadIndex);
+      } else {
+        float e0 = kNoFactor, e1 = 0.f;
+        if (contrib) oct_encode(dn, e0, e1);
+        float4 *f = a.gws.fac + 2 * (size_t)p;
+        __stcs(f, make_float4(dpre_s, dpre_g, dz[0], dz[1]));
+        __stcs(f + 1, make_float4(dz[2], to * (float)(a.tr.T - 1), e0, e1));
+      }
+    }
+  } else {
+    // lanes without a contribution get keys of their own (leaf ids are < 2^31)
+    const unsigned long long key =
+        contrib ? (((unsigned long long)leaf << 32) | __float_as_uint(to)) : (~0ull - (unsigned long long)lane);
+    const unsigned grp = __match_any_sync(kFull, key);
+    const bool leader = contrib && lane == __ffs(grp) - 1;
+    float F[3 * NY];
+#pragma unroll
+    for (int ch = 0; ch < 3; ++ch)
+#pragma unroll
+      for (int k = 0; k < NY; ++k) F[ch * NY + k] = dz[ch] * Y[k];
+    const int gmax = (int)__reduce_max_sync(kFull, contrib ? (unsigned)__popc(grp) : 1u);
+    unsigned rest = leader ? (grp & (grp - 1u)) : 0u;  // the leader's other members
+    for (int it = 1; it < gmax; ++it) {
+      const int src = rest ? __ffs(rest) - 1 : lane;
+      rest &= rest - 1u;
+      const bool add = src != lane;
+      const float xs = __shfl_sync(kFull, dpre_s, src);
+      const float xg = __shfl_sync(kFull, dpre_g, src);
+      if (add) {
+        dpre_s += xs;
+        dpre_g += xg;
+      }
+#pragma unroll
+      for (int k = 0; k < 3 * NY; ++k) {
+        const float x = __shfl_sync(kFull, F[k], src);
+        if (add) F[k] += x;
+      }
+    }
+    if (leader) scatter_gradient<KP, DEG>(a, rows, leaf, m.s.R, F, dpre_s, dpre_g);
+  }
+  __syncwarp();  // the shared results are rewritten by the next batch
 }
 
 // Whether a segment log was written by a forward over these rays.
@@ -413,63 +478,54 @@ cudaError_t launch_packet_order(const DevTree &tr, const DevRays &rays, const Sa
   return sort_packets_by_key(l, n_packets, tr.n_leaves, num_sms, s);
 }
 
-// Walking adjoint of one packet (ray i of this lane) that the segment log
-// does not hold: the forward packet kernel's structure (walk steps and sample
-// rounds decoupled through a per-lane queue), the walk stopped at the
-// forward's segment count.  Not inlined: its state does not add to the
+// Walking adjoint of one packet (ray i of this lane, when live) that the
+// segment log does not hold: the forward packet kernel's structure (walk steps
+// and batches decoupled through the packet's ring), each ray's walk stopped at
+// the forward's segment count.  Not inlined: its state does not add to the
 // registers of the replay, which most packets take.
 template <int KP, int DEG, typename E>
-__device__ __noinline__ void adjoint_walk_packet(const BwdArgs &a, long long i, unsigned present, int queue,
-                                                 int ready) {
+__device__ __noinline__ void adjoint_walk_packet(const BwdArgs &a, long long i, bool live, int ready) {
   extern __shared__ __align__(16) uint32_t smem[];
   const DevTree &tr = a.tr;
-  const int B = blockDim.x, tid = threadIdx.x;
-  float *my_rows = reinterpret_cast<float *>(smem) + tid;
-  const PathRef pr{smem + 2 * KP * B + tid, B};
-  uint32_t *q_leaf = smem + (2 * KP + path_words(tr)) * B + tid;
-  float *q_dt = reinterpret_cast<float *>(q_leaf + queue * B);
-  const SmemRows<KP> rows{my_rows, B};
+  const int lane = threadIdx.x & 31;
+  const PacketShared<KP> sh(smem);
+  const PathRef pr{sh.path, sh.stride};
   RayWalk w;
+  w.alive = false;
   AdjState st;
-  float dn[3], t;
-  const bool live = adjoint_setup(a, i, w, dn, t, st);
-  if (__ballot_sync(present, live) == 0) return;
-  if (live) rows_to_smem<KP>(tr, t * (float)(tr.T - 1), my_rows, B);
+  st.count = st.target = 0;
+  st.g[0] = st.g[1] = st.g[2] = 0.f;
+  float dn[3], t = 0.f;
+  live = live && adjoint_setup(a, i, w, dn, t, st);
+  if (!__any_sync(kFull, live)) return;
+  if (live) sh.put_ray(tr, dn, t * (float)(tr.T - 1), true);
   int walked = 0;  // segments found so far (the walk stops at the forward's count)
   bool walking = live && w.alive;
-  int qh = 0, qn = 0;
-  const int qmask = queue - 1;
+  int head = 0, count = 0;
   for (;;) {
-    if (walking && qn < queue) {
-      uint32_t leaf;
-      float t0, dt;
-      if (walk_step<true>(tr, w, leaf, t0, dt, pr)) {
-        const int slot = (qh + qn) & qmask;
-        q_leaf[slot * B] = leaf;
-        q_dt[slot * B] = dt;
-        ++qn;
-        ++walked;
-      }
+    uint32_t leaf = 0u;
+    float t0, dt = 0.f;
+    bool found = false;
+    if (walking) {
+      found = walk_step<true>(tr, w, leaf, t0, dt, pr);
+      walked += found ? 1 : 0;
       walking = w.alive && walked < st.target;
     }
-    const unsigned have = __ballot_sync(present, qn > 0);
-    const unsigned stepping = __ballot_sync(present, walking && qn < queue);
-    if (!have && !stepping) break;
-    const int active = __popc(__ballot_sync(present, walking || qn > 0));
-    if (stepping && __popc(have) < min(ready, active)) continue;
-    uint32_t leaf = kEmpty;
-    float dt = 0.f;
-    const bool has = qn > 0;
-    if (has) {
-      leaf = q_leaf[qh * B];
-      dt = q_dt[qh * B];
-      qh = (qh + 1) & qmask;
-      --qn;
-      ++st.count;
+    const unsigned finds = __ballot_sync(kFull, found);
+    if (found) {
+      const int slot = (head + count + __popc(finds & ((1u << lane) - 1u))) & (kRing - 1);
+      sh.ring[slot] = make_uint4(leaf, __float_as_uint(dt), 0u, lane);
     }
-    float Y[(DEG + 1) * (DEG + 1)];
-    sh_real<DEG>(dn, Y);
-    adjoint_round<KP, DEG, E>(a, rows, Y, leaf, dt, t, has, present, st);
+    count += __popc(finds);
+    if (count < ready && __any_sync(kFull, walking)) continue;
+    if (count == 0) break;
+    __syncwarp();
+    const int batch = min(count, 32);
+    const uint4 en = sh.ring[(head + lane) & (kRing - 1)];
+    head += batch;
+    count -= batch;
+    adjoint_batch<KP, DEG, E, false>(a, sh, en.x, __uint_as_float(en.y), (int)en.w & 31, lane < batch, lane < batch, t,
+                                    st);
   }
 }
 
@@ -477,65 +533,55 @@ __device__ __noinline__ void adjoint_walk_packet(const BwdArgs &a, long long i, 
 // segment log when the log holds the packet (no walk); other packets (all of
 // them without a log for these rays) take adjoint_walk_packet.
 template <int KP, int DEG, typename E>
-__global__ void __launch_bounds__(256, packet_min_blocks<E>()) render_bwd_packet_kernel(const __grid_constant__ BwdArgs a, int queue,
-                                                                int ready) {
+__global__ void __launch_bounds__(256, packet_min_blocks<E>()) render_bwd_packet_kernel(const __grid_constant__ BwdArgs a, int ready) {
   extern __shared__ __align__(16) uint32_t smem[];
   const DevTree &tr = a.tr;
-  const int B = blockDim.x, tid = threadIdx.x;
-  float *my_rows = reinterpret_cast<float *>(smem) + tid;
-  const SmemRows<KP> rows{my_rows, B};
+  const int lane = threadIdx.x & 31;
+  const PacketShared<KP> sh(smem);
   // warp w adjoins packet w, or with a valid log in key order (the atomic
   // scatter) the w-th packet of that order
   const long long n_packets = (a.rays.n + 31) >> 5;
-  const long long wp = ((long long)blockIdx.x * B + tid) >> 5;
+  const long long wp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (wp >= n_packets) return;
   const bool logged = a.log.n_chunks && log_matches(a.log, a.rays.n);
   const long long pk = logged && a.key_order ? (long long)min(__ldg(a.log.order + wp), (uint32_t)(n_packets - 1)) : wp;
-  const long long pos = (pk << 5) + (tid & 31);  // position; the ray is pos, or perm[pos] in a permuted log
-  const unsigned present = __ballot_sync(0xFFFFFFFFu, pos < a.rays.n);
-  if (pos >= a.rays.n) return;
-  const long long i =
-      logged && __ldg(a.log.header + 5) == 1u ? (long long)min(__ldg(a.log.perm + pos), (uint32_t)(a.rays.n - 1)) : pos;
+  const long long pos = (pk << 5) + lane;  // position; the ray is pos, or perm[pos] in a permuted log
+  bool live = pos < a.rays.n;
+  const long long i = live && logged && __ldg(a.log.header + 5) == 1u
+                          ? (long long)min(__ldg(a.log.perm + pos), (uint32_t)(a.rays.n - 1))
+                          : pos;
   const uint32_t head = logged ? __ldg(a.log.heads + pk) : kNoLog;  // warp-uniform
   if (head == kNoLog) {
-    adjoint_walk_packet<KP, DEG, E>(a, i, present, queue, ready);
+    adjoint_walk_packet<KP, DEG, E>(a, i, live, ready);
     return;
   }
   RayWalk w;
   AdjState st;
-  float dn[3], t;
-  const bool live = adjoint_setup(a, i, w, dn, t, st);
-  if (__ballot_sync(present, live) == 0) return;
-  if (live) rows_to_smem<KP>(tr, t * (float)(tr.T - 1), my_rows, B);
+  st.count = st.target = 0;
+  st.g[0] = st.g[1] = st.g[2] = 0.f;
+  float dn[3], t = 0.f;
+  live = live && adjoint_setup(a, i, w, dn, t, st);
+  if (!__any_sync(kFull, live)) return;
+  if (live) sh.put_ray(tr, dn, t * (float)(tr.T - 1), true);
+  __syncwarp();
   // replay the forward's shading rounds from its log: no walk
-  const int lane = tid & 31;
-  const float u = t * (float)(tr.T - 1);
+  const unsigned rays = __ballot_sync(kFull, live);
   uint32_t chunk = head;
   int round = 0;
-  while (__ballot_sync(present, live && st.count < st.target)) {
-    if (chunk >= a.log.n_chunks) {  // a log that does not belong to these rays
+  while (__any_sync(kFull, live && st.count < st.target)) {
+    if (chunk >= a.log.n_chunks) {  // the chain's end: a log that does not belong to these rays
       raise_status(tr, kStatusBadIndex);
       return;
     }
-    uint32_t leaf = kEmpty;
-    float dt = 0.f;
-    bool has = false;
     const size_t slot = ((size_t)chunk * kLogRounds + round) * 32 + lane;
-    if (live && st.count < st.target) {
-      leaf = __ldcs(a.log.leaf + slot);
-      if (leaf != kEmpty) {
-        ++st.count;
-        has = leaf < (uint32_t)tr.n_leaves;
-        if (has) dt = __ldcs(a.log.dt + slot);
-        else raise_status(tr, kStatusBadIndex);
-      }
-    }
-    // the harmonics of the ray's direction, per round rather than held
-    float Y[(DEG + 1) * (DEG + 1)];
-    sh_real<DEG>(dn, Y);
+    const uint32_t leaf = __ldcs(a.log.leaf + slot);
+    const float dt = __ldcs(a.log.dt + slot);
+    const int owner = (int)__ldcs(a.log.lane + slot) & 31;
+    const bool has = leaf != kEmpty && ((rays >> owner) & 1u), valid = has && leaf < (uint32_t)tr.n_leaves;
+    if (has && !valid) raise_status(tr, kStatusBadIndex);
     // chunks with room in the workspace: factors to the leaf's run; others: atomics
-    if (chunk < a.gws.cap_chunks) adjoint_round_gather<KP, DEG, E>(a, rows, Y, leaf, dt, u, dn, has, present, st);
-    else adjoint_round<KP, DEG, E>(a, rows, Y, leaf, dt, t, has, present, st);
+    if (chunk < a.gws.cap_chunks) adjoint_batch<KP, DEG, E, true>(a, sh, leaf, dt, owner, has, valid, t, st);
+    else adjoint_batch<KP, DEG, E, false>(a, sh, leaf, dt, owner, has, valid, t, st);
     if (++round == kLogRounds) {
       round = 0;
       chunk = __ldg(a.log.next + chunk);
@@ -852,7 +898,7 @@ static cudaError_t bwd_one(bool packet, const BwdArgs &a, const LaunchCfg &cfg, 
   if (!packet) {
     render_bwd_plain_kernel<KP, DEG, E><<<(unsigned)blocks, cfg.block, 0, s>>>(a);
   } else {
-    const size_t sm = smem_bytes(cfg.block, KP, cfg.queue, a.tr);
+    const size_t sm = smem_bytes(cfg.block, KP, a.tr);
     if (sm > 48 * 1024) {
       cudaError_t e = cudaFuncSetAttribute(render_bwd_packet_kernel<KP, DEG, E>,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
@@ -884,7 +930,7 @@ static cudaError_t bwd_one(bool packet, const BwdArgs &a, const LaunchCfg &cfg, 
       e = cudaMemcpyAsync(a.gws.cur, a.gws.off, (size_t)(nl + 1) * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s);
       if (e != cudaSuccess) return e;
     }
-    render_bwd_packet_kernel<KP, DEG, E><<<(unsigned)blocks, cfg.block, sm, s>>>(b, cfg.queue, cfg.ready);
+    render_bwd_packet_kernel<KP, DEG, E><<<(unsigned)blocks, cfg.block, sm, s>>>(b, cfg.ready);
     if (gather) {
       // the per-leaf sums over each leaf's run
       AdamArgs ad{};

@@ -45,14 +45,15 @@ __device__ __forceinline__ void write_miss(const DevOut &out, long long i) {
 // Packet forward kernel: one thread per ray, so each warp is a packet of 32
 // consecutive rays (an 8x4 pixel tile when the caller orders rays that way).
 // Walking and shading are decoupled: in every iteration of one warp-uniform
-// loop each lane takes at most one walk step and queues the occupied-leaf
-// segment it finds; the warp runs a shading round (each lane evaluates and
-// composites its oldest queued segment, in ray order) once `ready` lanes hold
-// one, or when no lane can step any further.  Lanes therefore do not wait at
-// every sample for the slowest searcher of the packet, and shading rounds run
-// nearly full.  Descents restart at the lowest common ancestor of successive
-// cells (path per thread in shared memory); basis rows and the queue live in
-// shared memory too.
+// loop each lane takes at most one walk step, and the occupied-leaf segments
+// found join the packet's ring.  Once `ready` segments wait, or no ray can step
+// any further, the warp shades a batch of up to 32 of them, one per lane
+// whichever rays they belong to, and each ray composites its own entries in
+// order (a shuffle of the seven values that compositing needs per entry).
+// Shading rounds therefore run full even where the packet's rays are uneven:
+// one long ray among finished ones shades up to 32 of its own segments at once.
+// Descents restart at the lowest common ancestor of successive cells (path per
+// thread in shared memory); basis rows and directions live in shared memory.
 // kShade: kShadeTree (the tree's records), kShadeSlice (a time slice,
 // a.slice), kShadeEdit (the tree's records with appearance edits, a.edits) or
 // kShadeAlpha (density only: the w_sigma part of each record is read, colour
@@ -60,123 +61,99 @@ __device__ __forceinline__ void write_miss(const DevOut &out, long long i) {
 // the full render).
 constexpr int kShadeTree = 0, kShadeSlice = 1, kShadeEdit = 2, kShadeAlpha = 3;
 template <int KP, int DEG, typename E, int kShade = kShadeTree>
-__device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pos, long long i, unsigned present,
-                                               int queue, int ready) {
+__device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, int ready) {
   extern __shared__ __align__(16) uint32_t smem[];
   const DevTree &tr = a.tr;
-  const int B = blockDim.x, tid = threadIdx.x;
-  float *my_rows = reinterpret_cast<float *>(smem) + tid;
-  const PathRef pr{smem + 2 * KP * B + tid, B};
-  uint32_t *q_leaf = smem + (2 * KP + path_words(tr)) * B + tid;
-  float *q_t0 = reinterpret_cast<float *>(q_leaf + queue * B);
-  float *q_dt = q_t0 + queue * B;
-  const SmemRows<KP> rows{my_rows, B};
-  float o[3], d[3], t, dn[3];
-  load_ray(a.rays, i, o, d, t);
-  RayWalk w;
-  const bool hit = walk_init(tr, o, d, w, dn);
-  if (!hit) write_miss(a.out, i);
+  const int lane = threadIdx.x & 31;
+  const PacketShared<KP> sh(smem);
+  const PathRef pr{sh.path, sh.stride};
+  const long long pos = (pk << 5) + lane;
   // i: the ray (its data and outputs); pos: its position (packet pos >> 5, lane)
-  if (a.log.n_chunks && (threadIdx.x & 31) == __ffs(present) - 1) {
-    a.log.key[pos >> 5] = kNoKey;
-    a.log.heads[pos >> 5] = kNoLog;  // until the packet's first chunk
+  const bool live = pos < a.rays.n;
+  const long long i = live && a.perm ? (long long)min(__ldg(a.perm + pos), (uint32_t)(a.rays.n - 1)) : pos;
+  float t = 0.f;
+  RayWalk w;
+  w.alive = false;
+  bool hit = false;
+  if (live) {
+    float o[3], d[3], dn[3];
+    load_ray(a.rays, i, o, d, t);
+    hit = walk_init(tr, o, d, w, dn);
+    if (hit) sh.put_ray(tr, dn, t * (float)(tr.T - 1), kShade != kShadeSlice);
+    else write_miss(a.out, i);
   }
-  if (__ballot_sync(present, hit) == 0) return;  // the whole packet missed the tree
-  if (hit && kShade != kShadeSlice) rows_to_smem<KP>(tr, t * (float)(tr.T - 1), my_rows, B);
+  if (a.log.n_chunks && lane == 0) {
+    a.log.key[pk] = kNoKey;
+    a.log.heads[pk] = kNoLog;  // until the packet's first chunk
+  }
+  if (!__any_sync(kFull, hit)) return;  // the whole packet missed the tree
   float T = 1.f, C0 = 0.f, C1 = 0.f, C2 = 0.f, A = 0.f, dnum = 0.f, tau = 0.f;
   int nseg = 0;
-  bool walking = hit && w.alive;
-  int qh = 0, qn = 0;  // queue head and length
-  const int qmask = queue - 1;
+  bool walking = hit && w.alive, dead = false;
+  int head = 0, count = 0;  // the ring's oldest entry and length (warp-uniform)
   // segment log of this packet (warp-uniform state): current chunk and round
-  const int lane = threadIdx.x & 31;
-  const long long pk = pos >> 5;
   bool logging = a.log.n_chunks != 0;
   uint32_t chunk = kNoLog;
   int round = kLogRounds;
   for (;;) {
-    if (walking && qn < queue) {
-      uint32_t leaf;
-      float t0, dt;
-      if (walk_step<true>(tr, w, leaf, t0, dt, pr)) {
-        const int slot = (qh + qn) & qmask;
-        q_leaf[slot * B] = leaf;
-        q_t0[slot * B] = t0;
-        q_dt[slot * B] = dt;
-        ++qn;
-        // the record is read when the segment's round comes: ask L2 for it now
-        if (kShade == kShadeSlice) slice_prefetch_l2(a.slice, a.slice_stride, DEG, leaf);
-        else if (kShade == kShadeAlpha) LeafRecord<KP, DEG, E>::prefetch_sigma_l2(tr, leaf);
-        else LeafRecord<KP, DEG, E>::prefetch_l2(tr, leaf);
-      }
+    uint32_t leaf = 0u;
+    float t0 = 0.f, dt = 0.f;
+    bool found = false;
+    if (walking) {
+      found = walk_step<true>(tr, w, leaf, t0, dt, pr);
       walking = w.alive;
     }
-    const unsigned have = __ballot_sync(present, qn > 0);
-    const unsigned stepping = __ballot_sync(present, walking && qn < queue);
-    if (!have && !stepping) break;
-    const int active = __popc(__ballot_sync(present, walking || qn > 0));
-    if (stepping && __popc(have) < min(ready, active)) continue;
-    if (logging) {
-      if (round == kLogRounds) {  // next chunk: one counter add per 8 rounds
-        const int leader = __ffs(present) - 1;
-        if (chunk == kNoLog) {  // the packet's sort key: the smallest leaf of its first round
-          const uint32_t k = __reduce_min_sync(present, qn > 0 ? q_leaf[qh * B] : kNoKey);
-          if (lane == leader) a.log.key[pk] = k;
-        }
-        uint32_t nc = kNoLog;
-        if (lane == leader) {
-          const unsigned long long c = atomicAdd(a.log.counter, 1ull);
-          if (c < a.log.n_chunks) {
-            nc = (uint32_t)c;
-            if (chunk == kNoLog) a.log.heads[pk] = nc;
-            else a.log.next[chunk] = nc;
-          } else {
-            a.log.heads[pk] = kNoLog;  // out of room: the adjoint walks this packet
-          }
-        }
-        nc = __shfl_sync(present, nc, leader);
-        logging = nc != kNoLog;
-        chunk = nc;
-        round = 0;
-      }
-      if (logging) {
-        const size_t slot = ((size_t)chunk * kLogRounds + round) * 32 + lane;
-        __stcs(a.log.leaf + slot, qn > 0 ? q_leaf[qh * B] : kEmpty);
-        __stcs(a.log.dt + slot, qn > 0 ? q_dt[qh * B] : 0.f);
-        ++round;
-      }
+    const unsigned finds = __ballot_sync(kFull, found);
+    if (found) {
+      const int slot = (head + count + __popc(finds & ((1u << lane) - 1u))) & (kRing - 1);
+      sh.ring[slot] = make_uint4(leaf, __float_as_uint(dt), __float_as_uint(w.t_base + fmaf(0.5f, dt, t0)), lane);
+      // the record is read when the segment's round comes: ask L2 for it now
+      if (kShade == kShadeSlice) slice_prefetch_l2(a.slice, a.slice_stride, DEG, leaf);
+      else if (kShade == kShadeAlpha) LeafRecord<KP, DEG, E>::prefetch_sigma_l2(tr, leaf);
+      else LeafRecord<KP, DEG, E>::prefetch_l2(tr, leaf);
     }
-    if (qn > 0) {
-      const uint32_t leaf = q_leaf[qh * B];
-      const float t0 = q_t0[qh * B], dt = q_dt[qh * B];
-      qh = (qh + 1) & qmask;
-      --qn;
-      float sigma, col[3];
-      // the harmonics of the ray's direction, formed per round rather than
-      // held through the walk (16 registers fewer across the loop)
-      float Y[(DEG + 1) * (DEG + 1)];
-      if (kShade != kShadeAlpha) sh_real<DEG>(dn, Y);
+    count += __popc(finds);
+    if (count < ready && __any_sync(kFull, walking)) continue;
+    if (count == 0) break;
+    // shade the oldest entries, one per lane
+    __syncwarp();
+    const int batch = min(count, 32);
+    const bool has = lane < batch;
+    const uint4 en = sh.ring[(head + lane) & (kRing - 1)];
+    head += batch;
+    count -= batch;
+    const int owner = (int)en.w & 31;
+    const float to = kShade == kShadeEdit ? __shfl_sync(kFull, t, owner) : 0.f;
+    float sd = 0.f, al = 0.f, ex = 1.f, col[3] = {0.f, 0.f, 0.f};
+    if (has) {
+      const uint32_t lf = en.x;
+      float sigma;
+      float dn[3], Y[(DEG + 1) * (DEG + 1)];
+      if (kShade != kShadeAlpha) {
+        sh.get_dir(owner, dn);
+        sh_real<DEG>(dn, Y);
+      }
       if constexpr (kShade == kShadeSlice) {
-        shade_slice<DEG>(a.slice, a.slice_stride, leaf, Y, a.act, sigma, col);
+        shade_slice<DEG>(a.slice, a.slice_stride, lf, Y, a.act, sigma, col);
       } else if constexpr (kShade == kShadeAlpha) {
         LeafRecord<KP, DEG, E> rec;
-        rec.load_sigma(tr, leaf);
-        sigma = fmaxf(pre_sigma_of<KP>(rows, rec), 0.f);
-        col[0] = col[1] = col[2] = 0.f;
+        rec.load_sigma(tr, lf);
+        sigma = fmaxf(pre_sigma_of<KP>(sh.rows_of(owner), rec), 0.f);
       } else {
         LeafRecord<KP, DEG, E> rec;
-        rec.load(tr, leaf);
+        rec.load(tr, lf);
         Sample<DEG> s;
-        eval_sample<KP, DEG, E>(tr, rows, Y, rec, a.act, s);
+        s.c[0] = s.c[1] = s.c[2] = 0.f;
+        eval_sample<KP, DEG, E>(tr, sh.rows_of(owner), Y, rec, a.act, s);
         sigma = s.sigma;
         col[0] = s.c[0];
         col[1] = s.c[1];
         col[2] = s.c[2];
         if constexpr (kShade == kShadeEdit) {
           // appearance edit of the voxel, active from its time t_d on
-          const float4 e0 = __ldg(reinterpret_cast<const float4 *>(a.edits) + 2 * (size_t)leaf);
-          const float4 e1 = __ldg(reinterpret_cast<const float4 *>(a.edits) + 2 * (size_t)leaf + 1);
-          if (t >= e1.x) {
+          const float4 e0 = __ldg(reinterpret_cast<const float4 *>(a.edits) + 2 * (size_t)lf);
+          const float4 e1 = __ldg(reinterpret_cast<const float4 *>(a.edits) + 2 * (size_t)lf + 1);
+          if (to >= e1.x) {
             if (e0.w >= 0.f) sigma = e0.w;
             col[0] = fmaf(a.edit_beta, e0.x - col[0], col[0]);
             col[1] = fmaf(a.edit_beta, e0.y - col[1], col[1]);
@@ -184,41 +161,84 @@ __device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pos, 
           }
         }
       }
-      ++nseg;
       if (sigma > 0.f) {
-        const float sd = sigma * dt;
-        const float e = __expf(-sd);
-        const float wgt = T * alpha_of(sd);
-        C0 = fmaf(wgt, col[0], C0);
-        C1 = fmaf(wgt, col[1], C1);
-        C2 = fmaf(wgt, col[2], C2);
+        sd = sigma * __uint_as_float(en.y);
+        ex = __expf(-sd);
+        al = alpha_of(sd);
+      } else {  // no contribution: weight 0, colour unused
+        col[0] = col[1] = col[2] = 0.f;
+      }
+    }
+    // each ray composites its entries of the batch, oldest first
+    unsigned mine = sh.entries_of_lane(has, owner);
+    if (dead) mine = 0u;
+    unsigned kept = 0u;
+    while (__any_sync(kFull, mine != 0u)) {
+      const int j = mine ? __ffs(mine) - 1 : lane;
+      const float x_al = __shfl_sync(kFull, al, j), x_ex = __shfl_sync(kFull, ex, j);
+      const float x_sd = __shfl_sync(kFull, sd, j), x_tm = __shfl_sync(kFull, __uint_as_float(en.z), j);
+      float x_c[3] = {0.f, 0.f, 0.f};
+      if (kShade != kShadeAlpha) {
+#pragma unroll
+        for (int ch = 0; ch < 3; ++ch) x_c[ch] = __shfl_sync(kFull, col[ch], j);
+      }
+      if (mine) {
+        mine &= mine - 1u;
+        kept |= 1u << j;
+        ++nseg;
+        const float wgt = T * x_al;
+        C0 = fmaf(wgt, x_c[0], C0);
+        C1 = fmaf(wgt, x_c[1], C1);
+        C2 = fmaf(wgt, x_c[2], C2);
         A += wgt;
-        dnum = fmaf(wgt, w.t_base + fmaf(0.5f, dt, t0), dnum);
-        tau += sd;
-        T *= e;
-        if (T < a.t_stop) {  // early termination: drop what is still queued
+        dnum = fmaf(wgt, x_tm, dnum);
+        tau += x_sd;
+        T *= x_ex;
+        if (T < a.t_stop) {  // early termination: drop what still waits
+          dead = true;
           walking = false;
-          qn = 0;
+          mine = 0u;
         }
       }
     }
-  }
-  if (logging) {
-    // slots that hold no segment read kEmpty, so that the log can be read
-    // slot by slot: the rounds of the last chunk that the packet did not
-    // reach, and in the packet past the last ray, the slots of its absent
-    // lanes in every chunk
-    for (int r = round; r < kLogRounds; ++r) a.log.leaf[((size_t)chunk * kLogRounds + r) * 32 + lane] = kEmpty;
-    if (present != 0xFFFFFFFFu && lane == __ffs(present) - 1) {
-      uint32_t c = a.log.heads[pk];
-      for (uint32_t k = 0; k < a.log.n_chunks && c < a.log.n_chunks; ++k) {
-        for (int j = 0; j < kLogRounds * 32; ++j)
-          if (!((present >> (j & 31)) & 1u)) a.log.leaf[(size_t)c * kLogRounds * 32 + j] = kEmpty;
-        if (c == chunk) break;
-        c = a.log.next[c];
+    if (logging) {
+      if (round == kLogRounds) {  // next chunk: one counter add per 8 rounds
+        if (chunk == kNoLog) {  // the packet's sort key: the smallest leaf of its first round
+          const uint32_t k = __reduce_min_sync(kFull, has ? en.x : kNoKey);
+          if (lane == 0) a.log.key[pk] = k;
+        }
+        uint32_t nc = kNoLog;
+        if (lane == 0) {
+          const unsigned long long c = atomicAdd(a.log.counter, 1ull);
+          if (c < a.log.n_chunks) {
+            nc = (uint32_t)c;
+            a.log.next[nc] = kNoLog;  // the chain's end until another chunk follows
+            if (chunk == kNoLog) a.log.heads[pk] = nc;
+            else a.log.next[chunk] = nc;
+          } else {
+            a.log.heads[pk] = kNoLog;  // out of room: the adjoint walks this packet
+          }
+        }
+        nc = __shfl_sync(kFull, nc, 0);
+        logging = nc != kNoLog;
+        chunk = nc;
+        round = 0;
+      }
+      if (logging) {
+        // the entries that were composited (a ray that ended drops its later ones)
+        const bool keep = (__reduce_or_sync(kFull, kept) >> lane) & 1u;
+        const size_t slot = ((size_t)chunk * kLogRounds + round) * 32 + lane;
+        __stcs(a.log.leaf + slot, keep ? en.x : kEmpty);
+        __stcs(a.log.dt + slot, keep ? __uint_as_float(en.y) : 0.f);
+        a.log.lane[slot] = (uint8_t)owner;
+        ++round;
       }
     }
   }
+  // slots that hold no segment read kEmpty, so that the log can be read slot
+  // by slot: the rounds of the last chunk that the packet did not reach
+  if (logging && chunk != kNoLog)
+    for (int r = round; r < kLogRounds; ++r) a.log.leaf[((size_t)chunk * kLogRounds + r) * 32 + lane] = kEmpty;
   if (!hit) return;
   if (kShade != kShadeAlpha) {
     __stcs(a.out.rgb + 3 * i + 0, C0);
@@ -235,7 +255,7 @@ __device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pos, 
 // warp takes the next 32-ray packet from the counter when it finishes one, so
 // a long ray holds up only its own warp, not the other warps of its block.
 template <int KP, int DEG, typename E, int kShade = kShadeTree>
-__global__ void __launch_bounds__(256, packet_min_blocks<E>()) render_packet_kernel(const __grid_constant__ FwdArgs a, int queue, int ready) {
+__global__ void __launch_bounds__(256, packet_min_blocks<E>()) render_packet_kernel(const __grid_constant__ FwdArgs a, int ready) {
   // one packet per warp of the grid, or (with a work counter) packets pulled
   // one after another until the counter passes the last
   const int lane = threadIdx.x & 31;
@@ -256,13 +276,7 @@ __global__ void __launch_bounds__(256, packet_min_blocks<E>()) render_packet_ker
   }
   while (pk < n_packets) {
     if (a.order) pk = (long long)min(__ldg(a.order + pk), (uint32_t)(n_packets - 1));
-    const long long pos = (pk << 5) + lane;
-    // lanes past the end sit the packet out; the others stay to its end
-    const unsigned present = __ballot_sync(0xFFFFFFFFu, pos < a.rays.n);
-    if (pos < a.rays.n) {
-      const long long i = a.perm ? (long long)min(__ldg(a.perm + pos), (uint32_t)(a.rays.n - 1)) : pos;
-      packet_forward<KP, DEG, E, kShade>(a, pos, i, present, queue, ready);
-    }
+    packet_forward<KP, DEG, E, kShade>(a, pk, ready);
     __syncwarp();
     if (!a.work) break;
     unsigned long long q = 0;
@@ -306,14 +320,14 @@ static cudaError_t fwd_one(bool packet, const FwdArgs &a, const LaunchCfg &cfg, 
   if (!packet) {
     render_plain_kernel<KP, DEG, E><<<(unsigned)blocks, cfg.block, 0, s>>>(a);
   } else {
-    const size_t sm = smem_bytes(cfg.block, KP, cfg.queue, a.tr);
+    const size_t sm = smem_bytes(cfg.block, KP, a.tr);
     if (sm > 48 * 1024) {
       cudaError_t e = cudaFuncSetAttribute(render_packet_kernel<KP, DEG, E>,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
       if (e != cudaSuccess) return e;
     }
     if (!a.work) {
-      render_packet_kernel<KP, DEG, E><<<(unsigned)blocks, cfg.block, sm, s>>>(a, cfg.queue, cfg.ready);
+      render_packet_kernel<KP, DEG, E><<<(unsigned)blocks, cfg.block, sm, s>>>(a, cfg.ready);
     } else {
       int per_sm = 0;
       cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, render_packet_kernel<KP, DEG, E>,
@@ -323,7 +337,7 @@ static cudaError_t fwd_one(bool packet, const FwdArgs &a, const LaunchCfg &cfg, 
       e = cudaMemsetAsync(a.work, 0, sizeof(unsigned long long), s);
       if (e != cudaSuccess) return e;
       render_packet_kernel<KP, DEG, E><<<(unsigned)(want < blocks ? want : blocks), cfg.block, sm, s>>>(
-          a, cfg.queue, cfg.ready);
+          a, cfg.ready);
     }
   }
   return cudaGetLastError();
@@ -556,7 +570,7 @@ static cudaError_t render_slice_one(const FwdArgs &a, const LaunchCfg &cfg, cuda
   const bool persistent = a.work != nullptr;
   cudaError_t e;
   if (persistent && (e = cudaMemsetAsync(a.work, 0, sizeof(unsigned long long), s)) != cudaSuccess) return e;
-  const size_t sm = smem_bytes(cfg.block, 8, cfg.queue, a.tr);
+  const size_t sm = smem_bytes(cfg.block, 8, a.tr);
   if (sm > 48 * 1024 && (e = cudaFuncSetAttribute(render_packet_kernel<8, DEG, __nv_bfloat16, kShadeSlice>,
                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
     return e;
@@ -569,7 +583,7 @@ static cudaError_t render_slice_one(const FwdArgs &a, const LaunchCfg &cfg, cuda
     const long long want = (long long)(per_sm > 0 ? per_sm : 1) * cfg.num_sms;
     if (want < grid) grid = want;
   }
-  render_packet_kernel<8, DEG, __nv_bfloat16, kShadeSlice><<<(unsigned)grid, cfg.block, sm, s>>>(a, cfg.queue, cfg.ready);
+  render_packet_kernel<8, DEG, __nv_bfloat16, kShadeSlice><<<(unsigned)grid, cfg.block, sm, s>>>(a, cfg.ready);
   return cudaGetLastError();
 }
 
@@ -681,7 +695,7 @@ template <int KP, int DEG, typename E>
 static cudaError_t edit_one(const FwdArgs &a, const LaunchCfg &cfg, cudaStream_t s) {
   if (a.rays.n == 0) return cudaSuccess;
   const long long blocks = (a.rays.n + cfg.block - 1) / cfg.block;
-  const size_t sm = smem_bytes(cfg.block, KP, cfg.queue, a.tr);
+  const size_t sm = smem_bytes(cfg.block, KP, a.tr);
   cudaError_t e;
   if (sm > 48 * 1024 && (e = cudaFuncSetAttribute(render_packet_kernel<KP, DEG, E, kShadeEdit>,
                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
@@ -696,7 +710,7 @@ static cudaError_t edit_one(const FwdArgs &a, const LaunchCfg &cfg, cudaStream_t
     if (want < grid) grid = want;
     if ((e = cudaMemsetAsync(a.work, 0, sizeof(unsigned long long), s)) != cudaSuccess) return e;
   }
-  render_packet_kernel<KP, DEG, E, kShadeEdit><<<(unsigned)grid, cfg.block, sm, s>>>(a, cfg.queue, cfg.ready);
+  render_packet_kernel<KP, DEG, E, kShadeEdit><<<(unsigned)grid, cfg.block, sm, s>>>(a, cfg.ready);
   return cudaGetLastError();
 }
 
@@ -708,12 +722,12 @@ template <int KP, int DEG, typename E>
 static cudaError_t alpha_one(const FwdArgs &a, const LaunchCfg &cfg, cudaStream_t s) {
   if (a.rays.n == 0) return cudaSuccess;
   const long long blocks = (a.rays.n + cfg.block - 1) / cfg.block;
-  const size_t sm = smem_bytes(cfg.block, KP, cfg.queue, a.tr);
+  const size_t sm = smem_bytes(cfg.block, KP, a.tr);
   cudaError_t e;
   if (sm > 48 * 1024 && (e = cudaFuncSetAttribute(render_packet_kernel<KP, DEG, E, kShadeAlpha>,
                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
     return e;
-  render_packet_kernel<KP, DEG, E, kShadeAlpha><<<(unsigned)blocks, cfg.block, sm, s>>>(a, cfg.queue, cfg.ready);
+  render_packet_kernel<KP, DEG, E, kShadeAlpha><<<(unsigned)blocks, cfg.block, sm, s>>>(a, cfg.ready);
   return cudaGetLastError();
 }
 
@@ -744,9 +758,9 @@ cudaError_t launch_render_edit(int KP, int DEG, DType dt, const FwdArgs &a, cons
   return cudaErrorNotSupported;
 }
 
-// Segment log decoder: ray i's composited segments are the entries of its
-// lane in its packet's chunks that hold a leaf, in round order, nseg[i] of
-// them.  count[i] = -1 when the ray's packet is not in the log (no log, a log
+// Segment log decoder: ray i's composited segments are the slots of its
+// packet's chunks that hold a leaf and name its lane, in slot order, nseg[i]
+// of them.  count[i] = -1 when the ray's packet is not in the log (no log, a log
 // of other rays, or a packet that did not fit); chunk links are checked
 // against the log's size.
 __global__ void __launch_bounds__(256) log_read_kernel(const SampleLog l, long long n, const int *nseg, int max_out,
@@ -766,25 +780,22 @@ __global__ void __launch_bounds__(256) log_read_kernel(const SampleLog l, long l
       c = 0;
     } else if (chunk != kNoLog) {
       c = 0;
-      int round = 0;
-      for (long long guard = 0; c < want && guard < (long long)l.n_chunks * kLogRounds; ++guard) {
+      for (uint32_t guard = 0; c < want && guard < l.n_chunks; ++guard) {
         if (chunk >= l.n_chunks) {
           c = -1;
           break;
         }
-        const size_t slot = ((size_t)chunk * kLogRounds + round) * 32 + (pos & 31);
-        const uint32_t lf = __ldg(l.leaf + slot);
-        if (lf != kEmpty) {
+        for (int k = 0; k < kLogRounds * 32 && c < want; ++k) {
+          const size_t slot = (size_t)chunk * kLogRounds * 32 + k;
+          const uint32_t lf = __ldg(l.leaf + slot);
+          if (lf == kEmpty || __ldg(l.lane + slot) != (pos & 31)) continue;
           if (c < max_out) {
             leaf[i * max_out + c] = (int)lf;
             chord[i * max_out + c] = __ldg(l.dt + slot);
           }
           ++c;
         }
-        if (++round == kLogRounds) {
-          round = 0;
-          chunk = __ldg(l.next + chunk);
-        }
+        if (c < want) chunk = __ldg(l.next + chunk);
       }
     }
   }
