@@ -1110,6 +1110,15 @@ neuvv_status prepare_compose(const neuvv_tree *const *trees, const float *transf
       }
     for (int r = 0; r < 3; ++r) p.trans[r] = (float)tr[r];
     p.scale = (float)std::sqrt(s2);
+    double r2 = 0.0;
+    for (int r = 0; r < 3; ++r) {
+      double c = tr[r];
+      for (int k = 0; k < 3; ++k) c += m[r][k] * 0.5 * ((double)t->bmin[k] + (double)t->bmax[k]);
+      p.ball[r] = (float)c;
+      const double half = 0.5 * ((double)t->bmax[r] - (double)t->bmin[r]);
+      r2 += s2 * half * half;
+    }
+    p.ball[3] = (float)r2;
     if (!std::isfinite(time_offsets[j])) return fail(NEUVV_ERR_INVALID_ARG, "time offset %d not finite", j);
     p.toff = time_offsets[j];
     for (int c = 0; c < 3; ++c) {

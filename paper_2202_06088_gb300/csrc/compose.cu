@@ -156,57 +156,117 @@ __device__ __forceinline__ bool walk_init_local(const DevTree &tr, const PrimPar
   return w.alive;
 }
 
+// Whether the line o + s d can reach the ball around a primitive's box: the
+// cheap test that most (ray, primitive) pairs end at.  The margins (2e-3 of
+// the squared radius, 1e-5 of the squared distance) are far above the FP32
+// error of the expression, so no ray that the exact test accepts is lost, and
+// a comparison with NaN accepts.
+__device__ __forceinline__ bool near_ball(const PrimParam &pp, const float o[3], const float d[3], float idd) {
+  const float m0 = pp.ball[0] - o[0], m1 = pp.ball[1] - o[1], m2 = pp.ball[2] - o[2];
+  const float mm = fmaf(m0, m0, fmaf(m1, m1, m2 * m2)), md = fmaf(m0, d[0], fmaf(m1, d[1], m2 * d[2]));
+  return !(mm - md * md * idd > fmaf(1.002f, pp.ball[3], 1e-5f * mm));
+}
+
+// One packet of 32 rays per warp.  The primitives are taken one after another
+// by the whole packet: each ray that meets the primitive walks its tree, the
+// segments found wait in the packet's ring and are shaded in full batches
+// (shade_batch), and the ray's sums become a layer.  A ray that misses a
+// primitive leaves no layer (it would have colour and alpha 0 and an infinite
+// depth, which change neither blending mode).
 template <int KP, int DEG, typename E>
-__global__ void __launch_bounds__(256) compose_kernel(const __grid_constant__ ComposeArgs a, int dynamic) {
+__global__ void __launch_bounds__(256, packet_min_blocks<KP, DEG, E>())
+    compose_kernel(const __grid_constant__ ComposeArgs a, int dynamic) {
+  extern __shared__ __align__(16) uint32_t smem[];
   const long long n = a.rays.n;
   const long long n_packets = (n + 31) >> 5;
   const long long stride = ((long long)gridDim.x * blockDim.x) >> 5;
   const int lane = threadIdx.x & 31;
+  const PacketShared<KP> sh(smem);
+  const Shading shading{a.act, a.t_stop, nullptr, 0, nullptr, 0.f};
   long long p;
   if (dynamic) {
     unsigned long long q = 0;
     if (lane == 0) q = atomicAdd(a.work, 1ull);
-    p = (long long)__shfl_sync(0xFFFFFFFFu, q, 0);
+    p = (long long)__shfl_sync(kFull, q, 0);
   } else {
     p = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   }
   while (p < n_packets) {
     const long long i = (p << 5) + lane;
-    if (i < n) {
-      float o[3], d[3], t;
-      load_ray(a.rays, i, o, d, t);
-      float Lc[kMaxPrims][3], La[kMaxPrims], Ld[kMaxPrims];
-      for (int j = 0; j < a.n_prims; ++j) {
-        const PrimParam &pp = a.prim[j];
-        const DevTree &tr = a.trees[pp.tree];
-        RayResult r;
-        clear(r);
-        RayWalk w;
-        float dn[3], t_base, dist_scale;
-        if (walk_init_local(tr, pp, o, d, w, dn, t_base, dist_scale)) {
+    const bool live = i < n;
+    float o[3] = {0.f, 0.f, 0.f}, d[3] = {0.f, 0.f, 0.f}, t = 0.f;
+    if (live) load_ray(a.rays, i, o, d, t);
+    const float idd = 1.f / fmaf(d[0], d[0], fmaf(d[1], d[1], d[2] * d[2]));
+    float Lc[kMaxPrims][3], La[kMaxPrims], Ld[kMaxPrims];
+    int n_layers = 0;
+    for (int j = 0; j < a.n_prims; ++j) {
+      const PrimParam &pp = a.prim[j];
+      const bool close = live && near_ball(pp, o, d, idd);
+      if (!__any_sync(kFull, close)) continue;
+      const DevTree &tr = a.trees[pp.tree];
+      RayWalk w;
+      w.alive = false;
+      float t_base = 0.f, dist_scale = 0.f;
+      bool hit = false;
+      if (close) {
+        float dn[3];
+        hit = walk_init_local(tr, pp, o, d, w, dn, t_base, dist_scale);
+        if (hit) {
           const float period = (float)(tr.T - 1);
           float u = fmodf(t * period + pp.toff, period);
           if (u < 0.f) u += period;
-          // world distance = t_base + (local distance) * |d| / |dl|
-          integrate_walk<KP, DEG, E>(tr, w, dn, u, a.t_stop, a.act, t_base, dist_scale, r);
+          sh.put_ray(tr, dn, u, true);
         }
-        Lc[j][0] = pp.tint[0] * r.C[0];
-        Lc[j][1] = pp.tint[1] * r.C[1];
-        Lc[j][2] = pp.tint[2] * r.C[2];
-        La[j] = r.A;
-        Ld[j] = depth_of(r);
       }
-      float I0, I1, I2, A, D;
+      if (!__any_sync(kFull, hit)) continue;
+      RayAccum acc;
+      bool walking = hit && w.alive;
+      int head = 0, count = 0;
+      for (;;) {
+        uint32_t leaf = 0u;
+        float t0 = 0.f, dt = 0.f;
+        bool found = false;
+        if (walking) {
+          found = walk_step(tr, w, leaf, t0, dt);
+          walking = w.alive;
+        }
+        const unsigned finds = __ballot_sync(kFull, found);
+        if (found) {
+          const int slot = (head + count + __popc(finds & ((1u << lane) - 1u))) & (kRing - 1);
+          // world distance = t_base + (local distance) * |d| / |dl|
+          sh.ring[slot] = make_uint4(leaf, __float_as_uint(dt),
+                                     __float_as_uint(fmaf(dist_scale, fmaf(0.5f, dt, t0), t_base)), lane);
+          LeafRecord<KP, DEG, E>::prefetch_l2(tr, leaf);
+        }
+        count += __popc(finds);
+        if (count < 32 && __any_sync(kFull, walking)) continue;
+        if (count == 0) break;
+        __syncwarp();
+        const int batch = min(count, 32);
+        const uint4 en = sh.ring[(head + lane) & (kRing - 1)];
+        head += batch;
+        count -= batch;
+        shade_batch<KP, DEG, E, kShadeTree>(tr, sh, shading, en, lane < batch, t, acc);
+        if (acc.dead) walking = false;
+      }
+      __syncwarp();  // the rays' shared data are rewritten for the next primitive
+      if (hit) {
+#pragma unroll
+        for (int ch = 0; ch < 3; ++ch) Lc[n_layers][ch] = pp.tint[ch] * acc.C[ch];
+        La[n_layers] = acc.A;
+        Ld[n_layers] = acc.depth();
+        ++n_layers;
+      }
+    }
+    if (live) {
+      float I0 = 0.f, I1 = 0.f, I2 = 0.f, A = 0.f, D = INFINITY;
       if (a.mode == 0) {
         // stable order by depth: repeatedly take the nearest unused layer
         unsigned int used = 0;
-        I0 = I1 = I2 = 0.f;
-        A = 0.f;
-        D = INFINITY;
-        for (int k = 0; k < a.n_prims; ++k) {
+        for (int k = 0; k < n_layers; ++k) {
           int best = -1;
           float bd = 0.f;
-          for (int j = 0; j < a.n_prims; ++j) {
+          for (int j = 0; j < n_layers; ++j) {
             if (used & (1u << j)) continue;
             if (best < 0 || Ld[j] < bd) {
               best = j;
@@ -222,12 +282,7 @@ __global__ void __launch_bounds__(256) compose_kernel(const __grid_constant__ Co
           D = fminf(D, Ld[best]);
         }
       } else {
-        I0 = Lc[0][0];
-        I1 = Lc[0][1];
-        I2 = Lc[0][2];
-        A = La[0];
-        D = Ld[0];
-        for (int j = 1; j < a.n_prims; ++j) {
+        for (int j = 0; j < n_layers; ++j) {
           if (Ld[j] <= D) {
             const float keep = 1.f - La[j];
             I0 = fmaf(keep, I0, Lc[j][0]);
@@ -253,7 +308,7 @@ __global__ void __launch_bounds__(256) compose_kernel(const __grid_constant__ Co
     if (dynamic) {
       unsigned long long q = 0;
       if (lane == 0) q = atomicAdd(a.work, 1ull);
-      p = (long long)__shfl_sync(0xFFFFFFFFu, q, 0);
+      p = (long long)__shfl_sync(kFull, q, 0);
     } else {
       p += stride;
     }
@@ -263,14 +318,19 @@ __global__ void __launch_bounds__(256) compose_kernel(const __grid_constant__ Co
 template <int KP, int DEG, typename E>
 static cudaError_t compose_one(const ComposeArgs &a, const LaunchCfg &cfg, cudaStream_t s) {
   if (a.rays.n == 0) return cudaSuccess;
+  const size_t sm = smem_bytes(cfg.block, KP, 0);
+  cudaError_t e;
+  if (sm > 48 * 1024 && (e = cudaFuncSetAttribute(compose_kernel<KP, DEG, E>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                  (int)sm)) != cudaSuccess)
+    return e;
   int grid = cfg.grid;
   if (grid <= 0) {
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, compose_kernel<KP, DEG, E>, cfg.block, 0);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, compose_kernel<KP, DEG, E>, cfg.block, sm);
     if (e != cudaSuccess) return e;
     grid = (per_sm > 0 ? per_sm : 1) * cfg.num_sms;
   }
-  compose_kernel<KP, DEG, E><<<grid, cfg.block, 0, s>>>(a, cfg.dynamic_queue);
+  compose_kernel<KP, DEG, E><<<grid, cfg.block, sm, s>>>(a, cfg.dynamic_queue);
   return cudaGetLastError();
 }
 

@@ -124,6 +124,7 @@ struct PrimParam {
   float minv_lo[9];  // ... and the remainders: minv + minv_lo is the inverse to ~2^-48
   float trans[3];    // translation of world-from-local
   float scale;     // s
+  float ball[4];   // world centre of the local box and the square of its circumscribed radius
   float toff;      // time offset, frames
   float tint[3];
   int tree;        // index into ComposeArgs::trees
@@ -252,15 +253,16 @@ constexpr int kRing = 64;
 constexpr int kPathWords = 16;
 __host__ __device__ inline int path_words(const DevTree &tr) { return tr.path_words; }
 constexpr int kPacketWords = 4 * kRing / 32 + 1 + 2 + 3;
-inline size_t smem_bytes(int block, int KP, const DevTree &tr) {
-  return (size_t)block * (kPacketWords + 2 * KP + path_words(tr)) * sizeof(float);
+inline size_t smem_bytes(int block, int KP, int path) {
+  return (size_t)block * (kPacketWords + 2 * KP + path) * sizeof(float);
 }
+inline size_t smem_bytes(int block, int KP, const DevTree &tr) { return smem_bytes(block, KP, path_words(tr)); }
 constexpr int kMaxQueue = 32;
 // Packet kernels are latency bound: two 256-thread blocks per SM (128
-// registers a thread) keep enough warps resident; FP32 records need the
-// registers of one block per SM instead.
-template <typename E>
-constexpr int packet_min_blocks() { return sizeof(E) == 4 ? 1 : 2; }
+// registers a thread) keep enough warps resident; the larger FP32 records need
+// the registers of one block per SM instead.
+template <int KP, int DEG, typename E>
+constexpr int packet_min_blocks() { return sizeof(E) == 4 && 2 * KP + 3 * n_hh(DEG) > 64 ? 1 : 2; }
 constexpr int kMaxDepth = 14;
 
 }  // namespace neuvv

@@ -123,6 +123,114 @@ struct PacketShared {
   }
 };
 
+// What a batch is shaded from: kShadeTree (the tree's records), kShadeSlice (a
+// time slice), kShadeEdit (the tree's records with appearance edits) or
+// kShadeAlpha (density only: the w_sigma part of each record is read, colour
+// is neither evaluated nor written; alpha, depth, tau and nseg are those of
+// the full render).
+constexpr int kShadeTree = 0, kShadeSlice = 1, kShadeEdit = 2, kShadeAlpha = 3;
+struct Shading {
+  int act;
+  float t_stop;
+  const float *slice;  // kShadeSlice: [n_leaves][slice_stride]
+  int slice_stride;
+  const float *edits;  // kShadeEdit: [n_leaves][8], blended by edit_beta
+  float edit_beta;
+};
+
+// A ray's composited sums.
+struct RayAccum {
+  float T = 1.f, C[3] = {0.f, 0.f, 0.f}, A = 0.f, dnum = 0.f, tau = 0.f;
+  int nseg = 0;
+  bool dead = false;  // ended early: its waiting entries are dropped
+  __device__ __forceinline__ float depth() const { return A >= 1e-4f ? dnum / A : INFINITY; }
+};
+
+// Shades one batch of a packet's ring, called by the whole warp: lane j holds
+// entry j (en; has: one of the batch) and evaluates it, whichever ray it
+// belongs to; each ray then composites its own entries, oldest first, into acc
+// (the values of an entry that compositing needs come by shuffle from its
+// lane).  t: the time of this lane's ray.  Returns the mask of the entries
+// this lane's ray composited.
+template <int KP, int DEG, typename E, int kShade>
+__device__ __forceinline__ unsigned shade_batch(const DevTree &tr, const PacketShared<KP> &sh, const Shading &p,
+                                                const uint4 en, bool has, float t, RayAccum &acc) {
+  const int lane = threadIdx.x & 31, owner = (int)en.w & 31;
+  const float to = kShade == kShadeEdit ? __shfl_sync(kFull, t, owner) : 0.f;
+  float sd = 0.f, al = 0.f, ex = 1.f, col[3] = {0.f, 0.f, 0.f};
+  if (has) {
+    const uint32_t leaf = en.x;
+    float sigma, dn[3], Y[(DEG + 1) * (DEG + 1)];
+    if (kShade != kShadeAlpha) {
+      sh.get_dir(owner, dn);
+      sh_real<DEG>(dn, Y);
+    }
+    if constexpr (kShade == kShadeSlice) {
+      shade_slice<DEG>(p.slice, p.slice_stride, leaf, Y, p.act, sigma, col);
+    } else if constexpr (kShade == kShadeAlpha) {
+      LeafRecord<KP, DEG, E> rec;
+      rec.load_sigma(tr, leaf);
+      sigma = fmaxf(pre_sigma_of<KP>(sh.rows_of(owner), rec), 0.f);
+    } else {
+      LeafRecord<KP, DEG, E> rec;
+      rec.load(tr, leaf);
+      Sample<DEG> s;
+      s.c[0] = s.c[1] = s.c[2] = 0.f;
+      eval_sample<KP, DEG, E>(tr, sh.rows_of(owner), Y, rec, p.act, s);
+      sigma = s.sigma;
+#pragma unroll
+      for (int ch = 0; ch < 3; ++ch) col[ch] = s.c[ch];
+      if constexpr (kShade == kShadeEdit) {
+        // appearance edit of the voxel, active from its time t_d on
+        const float4 e0 = __ldg(reinterpret_cast<const float4 *>(p.edits) + 2 * (size_t)leaf);
+        const float4 e1 = __ldg(reinterpret_cast<const float4 *>(p.edits) + 2 * (size_t)leaf + 1);
+        if (to >= e1.x) {
+          if (e0.w >= 0.f) sigma = e0.w;
+          col[0] = fmaf(p.edit_beta, e0.x - col[0], col[0]);
+          col[1] = fmaf(p.edit_beta, e0.y - col[1], col[1]);
+          col[2] = fmaf(p.edit_beta, e0.z - col[2], col[2]);
+        }
+      }
+    }
+    if (sigma > 0.f) {
+      sd = sigma * __uint_as_float(en.y);
+      ex = __expf(-sd);
+      al = alpha_of(sd);
+    } else {  // no contribution: weight 0, colour unused
+      col[0] = col[1] = col[2] = 0.f;
+    }
+  }
+  unsigned mine = sh.entries_of_lane(has, owner), kept = 0u;
+  if (acc.dead) mine = 0u;
+  while (__any_sync(kFull, mine != 0u)) {
+    const int j = mine ? __ffs(mine) - 1 : lane;
+    const float x_al = __shfl_sync(kFull, al, j), x_ex = __shfl_sync(kFull, ex, j);
+    const float x_sd = __shfl_sync(kFull, sd, j), x_tm = __shfl_sync(kFull, __uint_as_float(en.z), j);
+    float x_c[3] = {0.f, 0.f, 0.f};
+    if (kShade != kShadeAlpha) {
+#pragma unroll
+      for (int ch = 0; ch < 3; ++ch) x_c[ch] = __shfl_sync(kFull, col[ch], j);
+    }
+    if (mine) {
+      mine &= mine - 1u;
+      kept |= 1u << j;
+      ++acc.nseg;
+      const float wgt = acc.T * x_al;
+#pragma unroll
+      for (int ch = 0; ch < 3; ++ch) acc.C[ch] = fmaf(wgt, x_c[ch], acc.C[ch]);
+      acc.A += wgt;
+      acc.dnum = fmaf(wgt, x_tm, acc.dnum);
+      acc.tau += x_sd;
+      acc.T *= x_ex;
+      if (acc.T < p.t_stop) {
+        acc.dead = true;
+        mine = 0u;
+      }
+    }
+  }
+  return kept;
+}
+
 __device__ __forceinline__ float depth_of(const RayResult &r) { return r.A >= 1e-4f ? r.dnum / r.A : INFINITY; }
 
 }  // namespace neuvv

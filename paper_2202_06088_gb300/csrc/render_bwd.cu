@@ -533,7 +533,7 @@ __device__ __noinline__ void adjoint_walk_packet(const BwdArgs &a, long long i, 
 // segment log when the log holds the packet (no walk); other packets (all of
 // them without a log for these rays) take adjoint_walk_packet.
 template <int KP, int DEG, typename E>
-__global__ void __launch_bounds__(256, packet_min_blocks<E>()) render_bwd_packet_kernel(const __grid_constant__ BwdArgs a, int ready) {
+__global__ void __launch_bounds__(256, packet_min_blocks<KP, DEG, E>()) render_bwd_packet_kernel(const __grid_constant__ BwdArgs a, int ready) {
   extern __shared__ __align__(16) uint32_t smem[];
   const DevTree &tr = a.tr;
   const int lane = threadIdx.x & 31;

@@ -54,12 +54,6 @@ __device__ __forceinline__ void write_miss(const DevOut &out, long long i) {
 // one long ray among finished ones shades up to 32 of its own segments at once.
 // Descents restart at the lowest common ancestor of successive cells (path per
 // thread in shared memory); basis rows and directions live in shared memory.
-// kShade: kShadeTree (the tree's records), kShadeSlice (a time slice,
-// a.slice), kShadeEdit (the tree's records with appearance edits, a.edits) or
-// kShadeAlpha (density only: the w_sigma part of each record is read, colour
-// is neither evaluated nor written; alpha, depth, tau and nseg are those of
-// the full render).
-constexpr int kShadeTree = 0, kShadeSlice = 1, kShadeEdit = 2, kShadeAlpha = 3;
 template <int KP, int DEG, typename E, int kShade = kShadeTree>
 __device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, int ready) {
   extern __shared__ __align__(16) uint32_t smem[];
@@ -87,9 +81,9 @@ __device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, i
     a.log.heads[pk] = kNoLog;  // until the packet's first chunk
   }
   if (!__any_sync(kFull, hit)) return;  // the whole packet missed the tree
-  float T = 1.f, C0 = 0.f, C1 = 0.f, C2 = 0.f, A = 0.f, dnum = 0.f, tau = 0.f;
-  int nseg = 0;
-  bool walking = hit && w.alive, dead = false;
+  const Shading shading{a.act, a.t_stop, a.slice, a.slice_stride, a.edits, a.edit_beta};
+  RayAccum acc;
+  bool walking = hit && w.alive;
   int head = 0, count = 0;  // the ring's oldest entry and length (warp-uniform)
   // segment log of this packet (warp-uniform state): current chunk and round
   bool logging = a.log.n_chunks != 0;
@@ -122,85 +116,8 @@ __device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, i
     const uint4 en = sh.ring[(head + lane) & (kRing - 1)];
     head += batch;
     count -= batch;
-    const int owner = (int)en.w & 31;
-    const float to = kShade == kShadeEdit ? __shfl_sync(kFull, t, owner) : 0.f;
-    float sd = 0.f, al = 0.f, ex = 1.f, col[3] = {0.f, 0.f, 0.f};
-    if (has) {
-      const uint32_t lf = en.x;
-      float sigma;
-      float dn[3], Y[(DEG + 1) * (DEG + 1)];
-      if (kShade != kShadeAlpha) {
-        sh.get_dir(owner, dn);
-        sh_real<DEG>(dn, Y);
-      }
-      if constexpr (kShade == kShadeSlice) {
-        shade_slice<DEG>(a.slice, a.slice_stride, lf, Y, a.act, sigma, col);
-      } else if constexpr (kShade == kShadeAlpha) {
-        LeafRecord<KP, DEG, E> rec;
-        rec.load_sigma(tr, lf);
-        sigma = fmaxf(pre_sigma_of<KP>(sh.rows_of(owner), rec), 0.f);
-      } else {
-        LeafRecord<KP, DEG, E> rec;
-        rec.load(tr, lf);
-        Sample<DEG> s;
-        s.c[0] = s.c[1] = s.c[2] = 0.f;
-        eval_sample<KP, DEG, E>(tr, sh.rows_of(owner), Y, rec, a.act, s);
-        sigma = s.sigma;
-        col[0] = s.c[0];
-        col[1] = s.c[1];
-        col[2] = s.c[2];
-        if constexpr (kShade == kShadeEdit) {
-          // appearance edit of the voxel, active from its time t_d on
-          const float4 e0 = __ldg(reinterpret_cast<const float4 *>(a.edits) + 2 * (size_t)lf);
-          const float4 e1 = __ldg(reinterpret_cast<const float4 *>(a.edits) + 2 * (size_t)lf + 1);
-          if (to >= e1.x) {
-            if (e0.w >= 0.f) sigma = e0.w;
-            col[0] = fmaf(a.edit_beta, e0.x - col[0], col[0]);
-            col[1] = fmaf(a.edit_beta, e0.y - col[1], col[1]);
-            col[2] = fmaf(a.edit_beta, e0.z - col[2], col[2]);
-          }
-        }
-      }
-      if (sigma > 0.f) {
-        sd = sigma * __uint_as_float(en.y);
-        ex = __expf(-sd);
-        al = alpha_of(sd);
-      } else {  // no contribution: weight 0, colour unused
-        col[0] = col[1] = col[2] = 0.f;
-      }
-    }
-    // each ray composites its entries of the batch, oldest first
-    unsigned mine = sh.entries_of_lane(has, owner);
-    if (dead) mine = 0u;
-    unsigned kept = 0u;
-    while (__any_sync(kFull, mine != 0u)) {
-      const int j = mine ? __ffs(mine) - 1 : lane;
-      const float x_al = __shfl_sync(kFull, al, j), x_ex = __shfl_sync(kFull, ex, j);
-      const float x_sd = __shfl_sync(kFull, sd, j), x_tm = __shfl_sync(kFull, __uint_as_float(en.z), j);
-      float x_c[3] = {0.f, 0.f, 0.f};
-      if (kShade != kShadeAlpha) {
-#pragma unroll
-        for (int ch = 0; ch < 3; ++ch) x_c[ch] = __shfl_sync(kFull, col[ch], j);
-      }
-      if (mine) {
-        mine &= mine - 1u;
-        kept |= 1u << j;
-        ++nseg;
-        const float wgt = T * x_al;
-        C0 = fmaf(wgt, x_c[0], C0);
-        C1 = fmaf(wgt, x_c[1], C1);
-        C2 = fmaf(wgt, x_c[2], C2);
-        A += wgt;
-        dnum = fmaf(wgt, x_tm, dnum);
-        tau += x_sd;
-        T *= x_ex;
-        if (T < a.t_stop) {  // early termination: drop what still waits
-          dead = true;
-          walking = false;
-          mine = 0u;
-        }
-      }
-    }
+    const unsigned kept = shade_batch<KP, DEG, E, kShade>(tr, sh, shading, en, has, t, acc);
+    if (acc.dead) walking = false;  // early termination: what still waits is dropped
     if (logging) {
       if (round == kLogRounds) {  // next chunk: one counter add per 8 rounds
         if (chunk == kNoLog) {  // the packet's sort key: the smallest leaf of its first round
@@ -230,7 +147,7 @@ __device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, i
         const size_t slot = ((size_t)chunk * kLogRounds + round) * 32 + lane;
         __stcs(a.log.leaf + slot, keep ? en.x : kEmpty);
         __stcs(a.log.dt + slot, keep ? __uint_as_float(en.y) : 0.f);
-        a.log.lane[slot] = (uint8_t)owner;
+        a.log.lane[slot] = (uint8_t)en.w;
         ++round;
       }
     }
@@ -241,21 +158,20 @@ __device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, i
     for (int r = round; r < kLogRounds; ++r) a.log.leaf[((size_t)chunk * kLogRounds + r) * 32 + lane] = kEmpty;
   if (!hit) return;
   if (kShade != kShadeAlpha) {
-    __stcs(a.out.rgb + 3 * i + 0, C0);
-    __stcs(a.out.rgb + 3 * i + 1, C1);
-    __stcs(a.out.rgb + 3 * i + 2, C2);
+#pragma unroll
+    for (int ch = 0; ch < 3; ++ch) __stcs(a.out.rgb + 3 * i + ch, acc.C[ch]);
   }
-  __stcs(a.out.alpha + i, A);
-  if (a.out.depth) __stcs(a.out.depth + i, A >= 1e-4f ? dnum / A : INFINITY);
-  if (a.out.tau) __stcs(a.out.tau + i, tau);
-  if (a.out.nseg) __stcs(a.out.nseg + i, nseg);
+  __stcs(a.out.alpha + i, acc.A);
+  if (a.out.depth) __stcs(a.out.depth + i, acc.depth());
+  if (a.out.tau) __stcs(a.out.tau + i, acc.tau);
+  if (a.out.nseg) __stcs(a.out.nseg + i, acc.nseg);
 }
 
 // Packet forward kernel.  With a work counter the grid is persistent: each
 // warp takes the next 32-ray packet from the counter when it finishes one, so
 // a long ray holds up only its own warp, not the other warps of its block.
 template <int KP, int DEG, typename E, int kShade = kShadeTree>
-__global__ void __launch_bounds__(256, packet_min_blocks<E>()) render_packet_kernel(const __grid_constant__ FwdArgs a, int ready) {
+__global__ void __launch_bounds__(256, packet_min_blocks<KP, DEG, E>()) render_packet_kernel(const __grid_constant__ FwdArgs a, int ready) {
   // one packet per warp of the grid, or (with a work counter) packets pulled
   // one after another until the counter passes the last
   const int lane = threadIdx.x & 31;
