@@ -181,7 +181,9 @@ __global__ void __launch_bounds__(256, packet_min_blocks<KP, DEG, E>())
   const long long n_packets = (n + 31) >> 5;
   const long long stride = ((long long)gridDim.x * blockDim.x) >> 5;
   const int lane = threadIdx.x & 31;
-  const PacketShared<KP> sh(smem);
+  using Rec = LeafRecord<KP, DEG, E>;
+  using Shared = PacketShared<KP, Rec::kChunks>;
+  const Shared sh(smem);
   const Shading shading{a.act, a.t_stop, nullptr, 0, nullptr, 0.f};
   long long p;
   if (dynamic) {
@@ -222,6 +224,8 @@ __global__ void __launch_bounds__(256, packet_min_blocks<KP, DEG, E>())
       RayAccum acc;
       bool walking = hit && w.alive;
       int head = 0, count = 0;
+      uint4 en = make_uint4(0u, 0u, 0u, 0u);
+      bool has = false, pending = false;
       for (;;) {
         uint32_t leaf = 0u;
         float t0 = 0.f, dt = 0.f;
@@ -236,18 +240,35 @@ __global__ void __launch_bounds__(256, packet_min_blocks<KP, DEG, E>())
           // world distance = t_base + (local distance) * |d| / |dl|
           sh.ring[slot] = make_uint4(leaf, __float_as_uint(dt),
                                      __float_as_uint(fmaf(dist_scale, fmaf(0.5f, dt, t0), t_base)), lane);
-          LeafRecord<KP, DEG, E>::prefetch_l2(tr, leaf);
+          if (!Shared::kStaged) Rec::prefetch_l2(tr, leaf);
         }
         count += __popc(finds);
         if (count < 32 && __any_sync(kFull, walking)) continue;
-        if (count == 0) break;
+        // batches as in the packet forward: shaded one batch late when staged
         __syncwarp();
         const int batch = min(count, 32);
-        const uint4 en = sh.ring[(head + lane) & (kRing - 1)];
+        const bool next_has = lane < batch;
+        const uint4 next_en = sh.ring[(head + lane) & (kRing - 1)];
+        if (!Shared::kStaged) {
+          en = next_en;
+          has = next_has;
+          pending = batch > 0;
+        }
+        if (pending) {
+          if (Shared::kStaged) sh.staged_wait();
+          shade_batch<KP, DEG, E, kShadeTree>(tr, sh, shading, en, has, t, acc);
+          if (acc.dead) walking = false;
+        }
+        if (batch == 0) break;
         head += batch;
         count -= batch;
-        shade_batch<KP, DEG, E, kShadeTree>(tr, sh, shading, en, lane < batch, t, acc);
-        if (acc.dead) walking = false;
+        if (Shared::kStaged) {
+          __syncwarp();  // every lane has read its staged record
+          en = next_en;
+          has = next_has;
+          pending = true;
+          sh.stage_records(tr.rec, Rec::stride_bytes(tr), has ? en.x : 0u, batch);
+        }
       }
       __syncwarp();  // the rays' shared data are rewritten for the next primitive
       if (hit) {
@@ -318,7 +339,7 @@ __global__ void __launch_bounds__(256, packet_min_blocks<KP, DEG, E>())
 template <int KP, int DEG, typename E>
 static cudaError_t compose_one(const ComposeArgs &a, const LaunchCfg &cfg, cudaStream_t s) {
   if (a.rays.n == 0) return cudaSuccess;
-  const size_t sm = smem_bytes(cfg.block, KP, 0);
+  const size_t sm = smem_bytes(cfg.block, KP, LeafRecord<KP, DEG, E>::kChunks, 0);
   cudaError_t e;
   if (sm > 48 * 1024 && (e = cudaFuncSetAttribute(compose_kernel<KP, DEG, E>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                   (int)sm)) != cudaSuccess)

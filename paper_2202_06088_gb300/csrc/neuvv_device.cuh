@@ -611,7 +611,10 @@ struct LeafRecord {
   static constexpr int LEN = 2 * KP + 3 * NH;
   static constexpr int PV = Elem<E>::kPerVec;
   static constexpr int NV = (LEN + PV - 1) / PV;
+  static constexpr int kChunks = NV;  // 16-byte chunks of a storage record
   float w[NV * PV];
+
+  __device__ __forceinline__ static uint32_t stride_bytes(const DevTree &tr) { return (uint32_t)(tr.rec_stride * sizeof(E)); }
 
   __device__ __forceinline__ void load(const DevTree &tr, uint32_t leaf) {
     const uint4 *p = reinterpret_cast<const uint4 *>(static_cast<const E *>(tr.rec) + (size_t)leaf * tr.rec_stride);
@@ -621,10 +624,16 @@ struct LeafRecord {
 #pragma unroll
     for (int i = 0; i < NV; ++i) Elem<E>::unpack(raw[i], w + i * PV);
   }
-  // The same record from a copy in shared memory (a staged tile).
+  // The same record from a copy in shared memory (a staged tile), whole or the
+  // chunks that hold entries [lo, hi).
   __device__ __forceinline__ void load_shared(const uint4 *p) {
 #pragma unroll
     for (int i = 0; i < NV; ++i) Elem<E>::unpack(p[i], w + i * PV);
+  }
+  template <int LO, int HI>
+  __device__ __forceinline__ void load_part(const uint4 *p) {
+#pragma unroll
+    for (int i = LO / PV; i < (HI + PV - 1) / PV; ++i) Elem<E>::unpack(p[i], w + i * PV);
   }
   // Only the vectors that hold w_sigma and w_gamma.
   __device__ __forceinline__ void load_sigma_gamma(const DevTree &tr, uint32_t leaf) {
@@ -691,9 +700,11 @@ struct LeafRecord<KP, DEG, Fp8E4M3> {
   static constexpr int NH = n_hh(DEG);
   static constexpr int LEN = 2 * KP + 3 * NH;
   static constexpr int NV = (LEN + 15) / 16;
+  static constexpr int kChunks = NV + 1;
   uint4 raw[NV];  // codes, decoded where an entry is used
   float sc[3];    // group scales (powers of two)
 
+  __device__ __forceinline__ static uint32_t stride_bytes(const DevTree &tr) { return (uint32_t)tr.rec_stride; }
   __device__ __forceinline__ void load(const DevTree &tr, uint32_t leaf) {
     const uint4 *p = reinterpret_cast<const uint4 *>(static_cast<const unsigned char *>(tr.rec) +
                                                      (size_t)leaf * tr.rec_stride);
@@ -711,6 +722,15 @@ struct LeafRecord<KP, DEG, Fp8E4M3> {
     sc[0] = __uint_as_float(h.x);
     sc[1] = __uint_as_float(h.y);
     sc[2] = __uint_as_float(h.z);
+  }
+  template <int LO, int HI>
+  __device__ __forceinline__ void load_part(const uint4 *p) {
+    const uint4 h = p[0];
+    sc[0] = __uint_as_float(h.x);
+    sc[1] = __uint_as_float(h.y);
+    sc[2] = __uint_as_float(h.z);
+#pragma unroll
+    for (int i = LO / 16; i < (HI + 15) / 16; ++i) raw[i] = p[1 + i];
   }
   // The header and the code vectors that hold w_sigma and w_gamma.
   __device__ __forceinline__ void load_sigma_gamma(const DevTree &tr, uint32_t leaf) {
@@ -890,18 +910,38 @@ __device__ __forceinline__ float pre_sigma_of(const Rows &rows, const Rec &r) {
   return ((p4[0] + p4[1]) + (p4[2] + p4[3])) * r.scale_sigma();
 }
 
+// Where a sample's record comes from: loaded before the evaluation (Loaded),
+// or read from a staged copy in shared memory part by part just before each
+// part's use (FromShared).  The empty asm statements keep the compiler from
+// gathering all parts in registers first, which would spill the walk's state.
+struct Loaded {
+  template <int LO, int HI, typename Rec>
+  __device__ __forceinline__ void part(Rec &) const {}
+};
+struct FromShared {
+  const uint4 *p;
+  template <int LO, int HI, typename Rec>
+  __device__ __forceinline__ void part(Rec &r) const {
+    asm volatile("" ::: "memory");
+    r.template load_part<LO, HI>(p);
+  }
+};
+
 // Eq. project-sigma, Eq. project-gamma, Eq. HH-color-2 for one leaf.  When the
 // density is zero the sample cannot contribute and colour is not evaluated.
 // With kDz the gamma-derivative of each channel's pre-activation is formed
 // from the same inner sums sum_m w Y (the adjoint then needs no coefficient
 // after this call).
-template <int KP, int DEG, typename E, typename Rows, bool kDz = false>
-__device__ __forceinline__ void eval_sample(const DevTree &tr, const Rows &rows, const float *Y,
-                                            const LeafRecord<KP, DEG, E> &r, int act, Sample<DEG> &s) {
+template <int KP, int DEG, typename E, bool kDz = false, typename Rows, typename Source>
+__device__ __forceinline__ void eval_sample(const DevTree &tr, const Rows &rows, const float *Y, const Source &src,
+                                            LeafRecord<KP, DEG, E> &r, int act, Sample<DEG> &s) {
+  constexpr int NH = n_hh(DEG);
+  src.template part<0, KP>(r);
   const float ps = pre_sigma_of<KP>(rows, r);
   s.pre_sigma = ps;
   s.sigma = fmaxf(ps, 0.f);
   if (!(s.sigma > 0.f)) return;
+  src.template part<KP, 2 * KP>(r);
   float q4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
   for (int k = 0; k < KP; ++k) q4[k & 3] = fmaf(rows.B(k), r.gam(k), q4[k & 3]);
@@ -912,6 +952,9 @@ __device__ __forceinline__ void eval_sample(const DevTree &tr, const Rows &rows,
   hh_radial<DEG, kDz>(s.cg, s.sg, tr.hh_norm, s.R, dR);
 #pragma unroll
   for (int ch = 0; ch < 3; ++ch) {
+    if (ch == 0) src.template part<2 * KP, 2 * KP + NH>(r);
+    else if (ch == 1) src.template part<2 * KP + NH, 2 * KP + 2 * NH>(r);
+    else src.template part<2 * KP + 2 * NH, 2 * KP + 3 * NH>(r);
     float z = 0.f, u = 0.f;
 #pragma unroll
     for (int n = 0; n <= DEG; ++n)
@@ -933,8 +976,8 @@ __device__ __forceinline__ void eval_sample(const DevTree &tr, const Rows &rows,
 
 template <int KP, int DEG, typename E>
 __device__ __forceinline__ void eval_sample(const DevTree &tr, const RayConst<KP, DEG> &rc,
-                                            const LeafRecord<KP, DEG, E> &r, int act, Sample<DEG> &s) {
-  eval_sample<KP, DEG, E>(tr, RegRows<KP>{rc.a, rc.b}, rc.Y, r, act, s);
+                                            LeafRecord<KP, DEG, E> &r, int act, Sample<DEG> &s) {
+  eval_sample<KP, DEG, E>(tr, RegRows<KP>{rc.a, rc.b}, rc.Y, Loaded{}, r, act, s);
 }
 
 // ---------------------------------------------------------------------------

@@ -253,16 +253,27 @@ constexpr int kRing = 64;
 constexpr int kPathWords = 16;
 __host__ __device__ inline int path_words(const DevTree &tr) { return tr.path_words; }
 constexpr int kPacketWords = 4 * kRing / 32 + 1 + 2 + 3;
-inline size_t smem_bytes(int block, int KP, int path) {
-  return (size_t)block * (kPacketWords + 2 * KP + path) * sizeof(float);
+// Records of a batch staged in shared memory: 32 per warp, each of `chunks`
+// 16-byte chunks at an odd pitch, so that eight lanes reading one chunk of
+// their own records (a phase of a 16-byte load) hit distinct banks.  Smaller
+// records (K_pad 8, FP8) are read in place: staging them gains less than its
+// copies and the later shading cost (K_pad 8 BF16 composition 1044 against
+// 1100 us, a 128 x 128 FP32 view 78 against 83 us; K_pad 16 BF16 1080p view
+// 656 against 600 us).  So are records of more than 32 chunks (K_pad 32 in
+// FP32 with degree 3): eight warps' staging would not fit in an SM's shared
+// memory.
+constexpr int kMinStage = 16, kMaxStage = 32;
+__host__ __device__ constexpr bool staged(int chunks) { return chunks >= kMinStage && chunks <= kMaxStage; }
+__host__ __device__ constexpr int stage_pitch(int chunks) { return staged(chunks) ? (chunks | 1) : 0; }
+inline size_t smem_bytes(int block, int KP, int chunks, int path) {
+  return (size_t)block * (kPacketWords + 4 * stage_pitch(chunks) + 2 * KP + path) * sizeof(float);
 }
-inline size_t smem_bytes(int block, int KP, const DevTree &tr) { return smem_bytes(block, KP, path_words(tr)); }
 constexpr int kMaxQueue = 32;
 // Packet kernels are latency bound: two 256-thread blocks per SM (128
-// registers a thread) keep enough warps resident; the larger FP32 records need
-// the registers of one block per SM instead.
+// registers a thread) keep enough warps resident; records of more than
+// kMaxStage chunks need the registers of one block per SM instead.
 template <int KP, int DEG, typename E>
-constexpr int packet_min_blocks() { return sizeof(E) == 4 && 2 * KP + 3 * n_hh(DEG) > 64 ? 1 : 2; }
+constexpr int packet_min_blocks() { return LeafRecord<KP, DEG, E>::kChunks <= kMaxStage ? 2 : 1; }
 constexpr int kMaxDepth = 14;
 
 }  // namespace neuvv

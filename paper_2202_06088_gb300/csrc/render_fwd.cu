@@ -59,7 +59,9 @@ __device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, i
   extern __shared__ __align__(16) uint32_t smem[];
   const DevTree &tr = a.tr;
   const int lane = threadIdx.x & 31;
-  const PacketShared<KP> sh(smem);
+  constexpr int kChunks = shade_chunks<KP, DEG, E, kShade>();
+  using Shared = PacketShared<KP, kChunks>;
+  const Shared sh(smem);
   const PathRef pr{sh.path, sh.stride};
   const long long pos = (pk << 5) + lane;
   // i: the ray (its data and outputs); pos: its position (packet pos >> 5, lane)
@@ -85,6 +87,8 @@ __device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, i
   RayAccum acc;
   bool walking = hit && w.alive;
   int head = 0, count = 0;  // the ring's oldest entry and length (warp-uniform)
+  uint4 en = make_uint4(0u, 0u, 0u, 0u);  // this lane's entry of the batch to shade next
+  bool has = false, pending = false;
   // segment log of this packet (warp-uniform state): current chunk and round
   bool logging = a.log.n_chunks != 0;
   uint32_t chunk = kNoLog;
@@ -101,23 +105,30 @@ __device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, i
     if (found) {
       const int slot = (head + count + __popc(finds & ((1u << lane) - 1u))) & (kRing - 1);
       sh.ring[slot] = make_uint4(leaf, __float_as_uint(dt), __float_as_uint(w.t_base + fmaf(0.5f, dt, t0)), lane);
-      // the record is read when the segment's round comes: ask L2 for it now
-      if (kShade == kShadeSlice) slice_prefetch_l2(a.slice, a.slice_stride, DEG, leaf);
-      else if (kShade == kShadeAlpha) LeafRecord<KP, DEG, E>::prefetch_sigma_l2(tr, leaf);
-      else LeafRecord<KP, DEG, E>::prefetch_l2(tr, leaf);
+      if (!Shared::kStaged) {  // the record is read when the segment's batch comes: ask L2 for it now
+        if (kShade == kShadeSlice) slice_prefetch_l2(a.slice, a.slice_stride, DEG, leaf);
+        else if (kShade == kShadeAlpha) LeafRecord<KP, DEG, E>::prefetch_sigma_l2(tr, leaf);
+        else LeafRecord<KP, DEG, E>::prefetch_l2(tr, leaf);
+      }
     }
     count += __popc(finds);
     if (count < ready && __any_sync(kFull, walking)) continue;
-    if (count == 0) break;
-    // shade the oldest entries, one per lane
+    // the next batch: with staging its records are on their way while the
+    // rays walk on, and it is shaded when the one after it is complete
     __syncwarp();
     const int batch = min(count, 32);
-    const bool has = lane < batch;
-    const uint4 en = sh.ring[(head + lane) & (kRing - 1)];
-    head += batch;
-    count -= batch;
-    const unsigned kept = shade_batch<KP, DEG, E, kShade>(tr, sh, shading, en, has, t, acc);
-    if (acc.dead) walking = false;  // early termination: what still waits is dropped
+    const bool next_has = lane < batch;
+    const uint4 next_en = sh.ring[(head + lane) & (kRing - 1)];
+    if (!Shared::kStaged) {
+      en = next_en;
+      has = next_has;
+      pending = batch > 0;
+    }
+    unsigned kept = 0u;
+    if (pending) {
+      if (Shared::kStaged) sh.staged_wait();
+      kept = shade_batch<KP, DEG, E, kShade>(tr, sh, shading, en, has, t, acc);
+      if (acc.dead) walking = false;  // early termination: what still waits is dropped
     if (logging) {
       if (round == kLogRounds) {  // next chunk: one counter add per 8 rounds
         if (chunk == kNoLog) {  // the packet's sort key: the smallest leaf of its first round
@@ -150,6 +161,17 @@ __device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, i
         a.log.lane[slot] = (uint8_t)en.w;
         ++round;
       }
+    }
+    }
+    if (batch == 0) break;
+    head += batch;
+    count -= batch;
+    if (Shared::kStaged) {
+      __syncwarp();  // every lane has read its staged record
+      en = next_en;
+      has = next_has;
+      pending = true;
+      sh.stage_records(tr.rec, LeafRecord<KP, DEG, E>::stride_bytes(tr), has ? en.x : 0u, batch);
     }
   }
   // slots that hold no segment read kEmpty, so that the log can be read slot
@@ -236,7 +258,7 @@ static cudaError_t fwd_one(bool packet, const FwdArgs &a, const LaunchCfg &cfg, 
   if (!packet) {
     render_plain_kernel<KP, DEG, E><<<(unsigned)blocks, cfg.block, 0, s>>>(a);
   } else {
-    const size_t sm = smem_bytes(cfg.block, KP, a.tr);
+    const size_t sm = smem_bytes(cfg.block, KP, shade_chunks<KP, DEG, E, kShadeTree>(), path_words(a.tr));
     if (sm > 48 * 1024) {
       cudaError_t e = cudaFuncSetAttribute(render_packet_kernel<KP, DEG, E>,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
@@ -486,7 +508,7 @@ static cudaError_t render_slice_one(const FwdArgs &a, const LaunchCfg &cfg, cuda
   const bool persistent = a.work != nullptr;
   cudaError_t e;
   if (persistent && (e = cudaMemsetAsync(a.work, 0, sizeof(unsigned long long), s)) != cudaSuccess) return e;
-  const size_t sm = smem_bytes(cfg.block, 8, a.tr);
+  const size_t sm = smem_bytes(cfg.block, 8, shade_chunks<8, DEG, __nv_bfloat16, kShadeSlice>(), path_words(a.tr));
   if (sm > 48 * 1024 && (e = cudaFuncSetAttribute(render_packet_kernel<8, DEG, __nv_bfloat16, kShadeSlice>,
                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
     return e;
@@ -611,7 +633,7 @@ template <int KP, int DEG, typename E>
 static cudaError_t edit_one(const FwdArgs &a, const LaunchCfg &cfg, cudaStream_t s) {
   if (a.rays.n == 0) return cudaSuccess;
   const long long blocks = (a.rays.n + cfg.block - 1) / cfg.block;
-  const size_t sm = smem_bytes(cfg.block, KP, a.tr);
+  const size_t sm = smem_bytes(cfg.block, KP, shade_chunks<KP, DEG, E, kShadeEdit>(), path_words(a.tr));
   cudaError_t e;
   if (sm > 48 * 1024 && (e = cudaFuncSetAttribute(render_packet_kernel<KP, DEG, E, kShadeEdit>,
                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
@@ -638,7 +660,7 @@ template <int KP, int DEG, typename E>
 static cudaError_t alpha_one(const FwdArgs &a, const LaunchCfg &cfg, cudaStream_t s) {
   if (a.rays.n == 0) return cudaSuccess;
   const long long blocks = (a.rays.n + cfg.block - 1) / cfg.block;
-  const size_t sm = smem_bytes(cfg.block, KP, a.tr);
+  const size_t sm = smem_bytes(cfg.block, KP, shade_chunks<KP, DEG, E, kShadeAlpha>(), path_words(a.tr));
   cudaError_t e;
   if (sm > 48 * 1024 && (e = cudaFuncSetAttribute(render_packet_kernel<KP, DEG, E, kShadeAlpha>,
                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
