@@ -72,7 +72,7 @@ uint16_t bf16_bits(float f) {
   return (uint16_t)(u >> 16);
 }
 
-constexpr int kWorkSlots = 4;  // fwd, bwd, compose, spare
+constexpr int kWorkSlots = 8;  // 0: packet forward, 1: its triage's counts, 5: compose
 
 }  // namespace
 
@@ -81,6 +81,7 @@ struct neuvv_tree {
   uint32_t *child = nullptr;
   uint32_t *bricks = nullptr;
   uint32_t *coarse = nullptr;
+  uint32_t *queue = nullptr;   // triage of the packet forward: [kQueueEntries] (trees with a brick map)
   int brick_level = 0, brick_first = 0, brick_count = 0;
   void *rec = nullptr;
   float *master = nullptr, *m = nullptr, *v = nullptr;
@@ -680,6 +681,7 @@ neuvv_status neuvv_tree_create(const neuvv_tree_desc *desc, neuvv_tree **out) {
         brick_empty_boxes(br, boxed, map, nc, d.depth);
         br.swap(boxed);
         coarse_empty_boxes(occ, dist, nc, map);
+        NEUVV_TRY(cudaMalloc(&t->queue, kQueueEntries * 4), "cudaMalloc(packet queue)");
         NEUVV_TRY(cudaMalloc(&t->coarse, n3 * 4), "cudaMalloc(brick map)");
         NEUVV_TRY(cudaMemcpy(t->coarse, map.data(), n3 * 4, cudaMemcpyHostToDevice), "copy brick map");
       }
@@ -701,6 +703,7 @@ neuvv_status neuvv_tree_destroy(neuvv_tree *t) {
   cudaFree(t->child);
   cudaFree(t->bricks);
   cudaFree(t->coarse);
+  cudaFree(t->queue);
   cudaFree(t->m);
   cudaFree(t->v);
   cudaFree(t->A);
@@ -805,6 +808,7 @@ neuvv_status neuvv_render(const neuvv_tree *t, const neuvv_rays *rays, float tim
   const bool packet = opts->kernel != NEUVV_KERNEL_PLAIN;
   const LaunchCfg &cfg = packet ? t->packet : t->plain;
   a.work = packet && cfg.dynamic_queue ? t->work + 0 : nullptr;
+  a.queue = t->queue;
   int64_t chunk_bytes = 0;
   a.log = packet ? log_view(out->log, out->log_bytes, rays->n, &chunk_bytes) : log_view(nullptr, 0, 0);
   a.slice = nullptr;
@@ -814,7 +818,7 @@ neuvv_status neuvv_render(const neuvv_tree *t, const neuvv_rays *rays, float tim
   a.order = nullptr;
   cudaError_t e;
   if (a.log.n_chunks) {
-    e = cudaMemsetAsync(a.log.counter, 0, sizeof(unsigned long long), st);
+    e = cudaMemsetAsync(a.log.counter, 0, 64, st);  // the whole header; the kernels fill it
     if (e != cudaSuccess) return cuda_fail(e, "reset log");
     if (cfg.order == 1 && a.work) {
       // persistent warps take the packets in the order of the regions they reach
@@ -907,6 +911,7 @@ neuvv_status neuvv_render_slice(const neuvv_tree *t, const float *slice, int32_t
   a.act = opts->color_act;
   const LaunchCfg &cfg = t->packet;
   a.work = cfg.dynamic_queue ? t->work + 0 : nullptr;
+  a.queue = t->queue;
   a.log = log_view(nullptr, 0, 0);
   a.slice = slice;
   a.slice_stride = slice_stride;
@@ -1148,7 +1153,7 @@ neuvv_status neuvv_compose(const neuvv_tree *const *trees, const float *transfor
   if (rays->n == 0) return NEUVV_OK;
   DeviceGuard g(t0->info.device);
   cudaStream_t st = (cudaStream_t)stream;
-  a.work = t0->work + 2;
+  a.work = t0->work + 5;
   const LaunchCfg &cfg = t0->compose;
   if (cfg.dynamic_queue) {
     cudaError_t e = cudaMemsetAsync(a.work, 0, sizeof(unsigned long long), st);
@@ -1236,7 +1241,7 @@ neuvv_status neuvv_pick(const neuvv_tree *t, const neuvv_rays *rays, float time,
   std::memset(&a, 0, sizeof a);
   a.tr = dev_tree(t);
   a.rays = dev_rays(rays, time);
-  cudaError_t e = launch_pick(t->info.K_pad, t->info.hh_degree, (DType)t->info.dtype, a, threshold, leaf,
+  cudaError_t e = launch_pick(t->info.K_pad, t->info.hh_degree, (DType)t->info.dtype, a, threshold, leaf, t->packet,
                               (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "pick launch");
   return NEUVV_OK;
@@ -1280,6 +1285,7 @@ neuvv_status neuvv_render_edit(const neuvv_tree *t, const neuvv_rays *rays, floa
   a.act = opts->color_act;
   const LaunchCfg &cfg = t->packet;
   a.work = cfg.dynamic_queue ? t->work + 0 : nullptr;
+  a.queue = t->queue;
   a.log = log_view(nullptr, 0, 0);
   a.edits = edits;
   a.edit_beta = beta;

@@ -183,6 +183,14 @@ __device__ __forceinline__ bool box_interval(const DevTree &tr, const float o[3]
   return hit && s_in < s_out;
 }
 
+// Whether a ray given in the tree's own frame meets the tree's box, and its
+// parameters there.
+__device__ __forceinline__ bool ray_meets_box(const DevTree &tr, const float o[3], const float d[3], float &s_in,
+                                              float &s_out) {
+  int ax;
+  return sqrtf(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]) > 0.f && box_interval(tr, o, d, s_in, s_out, ax);
+}
+
 // Starts the walk at point p + pl of the tree's frame (inside the box; on
 // the entry face when the ray comes from outside; pl the part of the point
 // below p's FP32 precision) along the unit direction dn.

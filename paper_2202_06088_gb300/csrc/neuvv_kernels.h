@@ -35,7 +35,8 @@ constexpr int kLogRounds = 8;
 constexpr uint32_t kNoLog = 0xFFFFFFFFu;
 struct SampleLog {
   unsigned long long *counter;
-  uint32_t *header;   // [0] n_chunks, [1] rounds, [2..3] n_rays, [4] valid, [5] permuted
+  uint32_t *header;   // [0] n_chunks, [1] rounds, [2..3] n_rays, [4] valid, [5] permuted, [6..7] n_live:
+                      // positions from n_live on hold rays that miss the tree's box ([8] counts them)
   uint32_t *perm;     // [n_rays] ray of each position (when permuted)
   uint32_t *heads;    // [n_packets]
   uint32_t *key;      // [n_packets] first leaf the packet shaded (kNoKey: none)
@@ -66,7 +67,22 @@ struct FwdArgs {
   float edit_beta;           // colour blend weight of an active edit
   const uint32_t *order;     // persistent warps take packets in this order (null: packet index order)
   const uint32_t *perm;      // ray at each position (null: position = ray)
+  uint32_t *queue;           // tree-owned list [kQueueEntries] of the packet triage (null: none)
+  const uint32_t *list;      // parts to run (part_entry): list[0 .. counts[0]) then list[kQueueEntries - 1]
+  const uint32_t *counts;    //   downwards, counts[1] of them (null: all packets)
+  int split;                 // without a list: log2 of the parts each packet is run in
+  const uint32_t *n_live;    // rays at the first *n_live positions only (null: all)
 };
+// A packet may be run in 1, 2 or 4 parts, each a warp holding 32 / parts of its
+// rays: batches are full whatever rays they come from, so a part's shading
+// costs its share only, and a long packet no longer outlasts the others.
+constexpr int kMaxSplit = 2;  // log2
+// Entries of the triage's list, and the packets it takes (8.4 M rays) when
+// each may be listed in four parts.
+constexpr long long kQueueEntries = 1 << 20, kQueuePackets = kQueueEntries >> kMaxSplit;
+__host__ __device__ constexpr uint32_t part_entry(uint32_t packet, int split, int part) {
+  return packet | ((uint32_t)split << 20) | ((uint32_t)part << 24);
+}
 
 // Workspace of the leaf-major adjoint (owned by the tree; fac has one
 // 32-byte record per slot of the first cap_chunks chunks of a segment log).
@@ -214,7 +230,8 @@ cudaError_t launch_render_bwd(int KP, int DEG, DType dt, bool packet, const BwdA
                               cudaStream_t s, const AdamArgs *adam = nullptr, bool *fused = nullptr);
 cudaError_t launch_compose(int KP, int DEG, DType dt, const ComposeArgs &a, const LaunchCfg &cfg, cudaStream_t s);
 cudaError_t launch_trace(const TraceArgs &a, cudaStream_t s);
-cudaError_t launch_pick(int KP, int DEG, DType dt, const FwdArgs &a, float threshold, int *leaf_out, cudaStream_t s);
+cudaError_t launch_pick(int KP, int DEG, DType dt, const FwdArgs &a, float threshold, int *leaf_out,
+                        const LaunchCfg &cfg, cudaStream_t s);
 cudaError_t launch_paint(const int *leaf, const float *color, long long n, long long n_leaves, float *accum,
                          float sigma_d, float t_d, float *edits, cudaStream_t s);
 cudaError_t launch_render_edit(int KP, int DEG, DType dt, const FwdArgs &a, const LaunchCfg &cfg, cudaStream_t s);

@@ -170,12 +170,14 @@ struct PacketShared {
 // time slice), kShadeEdit (the tree's records with appearance edits) or
 // kShadeAlpha (density only: the w_sigma part of each record is read, colour
 // is neither evaluated nor written; alpha, depth, tau and nseg are those of
-// the full render).
-constexpr int kShadeTree = 0, kShadeSlice = 1, kShadeEdit = 2, kShadeAlpha = 3;
+// the full render) or kShadePick (density only: the leaf at which the ray's
+// opacity first reaches t_stop, in RayAccum::nseg).
+constexpr int kShadeTree = 0, kShadeSlice = 1, kShadeEdit = 2, kShadeAlpha = 3, kShadePick = 4;
+__host__ __device__ constexpr bool density_only(int shade) { return shade == kShadeAlpha || shade == kShadePick; }
 template <int KP, int DEG, typename E, int kShade>
 __host__ __device__ constexpr int shade_chunks() {
   // slice rows are small, and a density-only batch reads few chunks: in place
-  return kShade == kShadeSlice || kShade == kShadeAlpha ? 0 : LeafRecord<KP, DEG, E>::kChunks;
+  return kShade == kShadeSlice || density_only(kShade) ? 0 : LeafRecord<KP, DEG, E>::kChunks;
 }
 struct Shading {
   int act;
@@ -210,13 +212,13 @@ __device__ __forceinline__ unsigned shade_batch(const DevTree &tr, const Sh &sh,
   if (has) {
     const uint32_t leaf = en.x;
     float sigma, dn[3], Y[(DEG + 1) * (DEG + 1)];
-    if (kShade != kShadeAlpha) {
+    if (!density_only(kShade)) {
       sh.get_dir(owner, dn);
       sh_real<DEG>(dn, Y);
     }
     if constexpr (kShade == kShadeSlice) {
       shade_slice<DEG>(p.slice, p.slice_stride, leaf, Y, p.act, sigma, col);
-    } else if constexpr (kShade == kShadeAlpha) {
+    } else if constexpr (density_only(kShade)) {
       LeafRecord<KP, DEG, E> rec;
       rec.load_sigma(tr, leaf);
       sigma = fmaxf(pre_sigma_of<KP>(sh.rows_of(owner), rec), 0.f);
@@ -245,7 +247,9 @@ __device__ __forceinline__ unsigned shade_batch(const DevTree &tr, const Sh &sh,
         }
       }
     }
-    if (sigma > 0.f) {
+    if constexpr (kShade == kShadePick) {
+      sd = sigma;
+    } else if (sigma > 0.f) {
       sd = sigma * __uint_as_float(en.y);
       ex = __expf(-sd);
       al = alpha_of(sd);
@@ -255,12 +259,29 @@ __device__ __forceinline__ unsigned shade_batch(const DevTree &tr, const Sh &sh,
   }
   unsigned mine = sh.entries_of_lane(has, owner), kept = 0u;
   if (acc.dead) mine = 0u;
+  if constexpr (kShade == kShadePick) {
+    while (__any_sync(kFull, mine != 0u)) {
+      const int j = mine ? __ffs(mine) - 1 : lane;
+      const float x_sigma = __shfl_sync(kFull, sd, j), x_dt = __shfl_sync(kFull, __uint_as_float(en.y), j);
+      const uint32_t x_leaf = __shfl_sync(kFull, en.x, j);
+      if (mine) {
+        mine &= mine - 1u;
+        acc.tau = fmaf(x_sigma, x_dt, acc.tau);
+        if (-expm1f(-acc.tau) >= p.t_stop) {
+          acc.nseg = (int)x_leaf;
+          acc.dead = true;
+          mine = 0u;
+        }
+      }
+    }
+    return 0u;
+  }
   while (__any_sync(kFull, mine != 0u)) {
     const int j = mine ? __ffs(mine) - 1 : lane;
     const float x_al = __shfl_sync(kFull, al, j), x_ex = __shfl_sync(kFull, ex, j);
     const float x_sd = __shfl_sync(kFull, sd, j), x_tm = __shfl_sync(kFull, __uint_as_float(en.z), j);
     float x_c[3] = {0.f, 0.f, 0.f};
-    if (kShade != kShadeAlpha) {
+    if (!density_only(kShade)) {
 #pragma unroll
       for (int ch = 0; ch < 3; ++ch) x_c[ch] = __shfl_sync(kFull, col[ch], j);
     }

@@ -580,6 +580,8 @@ __global__ void __launch_bounds__(256, LeafRecord<KP, DEG, E>::kChunks <= 20 ? 2
   const bool logged = a.log.n_chunks && log_matches(a.log, a.rays.n);
   const long long pk = logged && a.key_order ? (long long)min(__ldg(a.log.order + wp), (uint32_t)(n_packets - 1)) : wp;
   const long long pos = (pk << 5) + lane;  // position; the ray is pos, or perm[pos] in a permuted log
+  // positions past the log's live rays hold rays that missed the tree
+  if (logged && (pk << 5) >= ((long long)__ldg(a.log.header + 7) << 32 | __ldg(a.log.header + 6))) return;
   bool live = pos < a.rays.n;
   const long long i = live && logged && __ldg(a.log.header + 5) == 1u
                           ? (long long)min(__ldg(a.log.perm + pos), (uint32_t)(a.rays.n - 1))

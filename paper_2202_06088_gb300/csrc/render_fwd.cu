@@ -55,7 +55,8 @@ __device__ __forceinline__ void write_miss(const DevOut &out, long long i) {
 // Descents restart at the lowest common ancestor of successive cells (path per
 // thread in shared memory); basis rows and directions live in shared memory.
 template <int KP, int DEG, typename E, int kShade = kShadeTree>
-__device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, int ready) {
+__device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, int split, int part, long long n_live,
+                                               int ready) {
   extern __shared__ __align__(16) uint32_t smem[];
   const DevTree &tr = a.tr;
   const int lane = threadIdx.x & 31;
@@ -63,9 +64,10 @@ __device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, i
   using Shared = PacketShared<KP, kChunks>;
   const Shared sh(smem);
   const PathRef pr{sh.path, sh.stride};
-  const long long pos = (pk << 5) + lane;
+  // the warp holds 32 >> split of the packet's rays, in its first lanes
+  const long long pos = (pk << 5) + (part << (5 - split)) + lane;
   // i: the ray (its data and outputs); pos: its position (packet pos >> 5, lane)
-  const bool live = pos < a.rays.n;
+  const bool live = lane < (32 >> split) && pos < n_live;
   const long long i = live && a.perm ? (long long)min(__ldg(a.perm + pos), (uint32_t)(a.rays.n - 1)) : pos;
   float t = 0.f;
   RayWalk w;
@@ -76,6 +78,7 @@ __device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, i
     load_ray(a.rays, i, o, d, t);
     hit = walk_init(tr, o, d, w, dn);
     if (hit) sh.put_ray(tr, dn, t * (float)(tr.T - 1), kShade != kShadeSlice);
+    else if (kShade == kShadePick) __stcs(a.out.nseg + i, -1);
     else write_miss(a.out, i);
   }
   if (a.log.n_chunks && lane == 0) {
@@ -85,6 +88,7 @@ __device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, i
   if (!__any_sync(kFull, hit)) return;  // the whole packet missed the tree
   const Shading shading{a.act, a.t_stop, a.slice, a.slice_stride, a.edits, a.edit_beta};
   RayAccum acc;
+  if (kShade == kShadePick) acc.nseg = -1;
   bool walking = hit && w.alive;
   int head = 0, count = 0;  // the ring's oldest entry and length (warp-uniform)
   uint4 en = make_uint4(0u, 0u, 0u, 0u);  // this lane's entry of the batch to shade next
@@ -107,7 +111,7 @@ __device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, i
       sh.ring[slot] = make_uint4(leaf, __float_as_uint(dt), __float_as_uint(w.t_base + fmaf(0.5f, dt, t0)), lane);
       if (!Shared::kStaged) {  // the record is read when the segment's batch comes: ask L2 for it now
         if (kShade == kShadeSlice) slice_prefetch_l2(a.slice, a.slice_stride, DEG, leaf);
-        else if (kShade == kShadeAlpha) LeafRecord<KP, DEG, E>::prefetch_sigma_l2(tr, leaf);
+        else if (density_only(kShade)) LeafRecord<KP, DEG, E>::prefetch_sigma_l2(tr, leaf);
         else LeafRecord<KP, DEG, E>::prefetch_l2(tr, leaf);
       }
     }
@@ -179,6 +183,10 @@ __device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, i
   if (logging && chunk != kNoLog)
     for (int r = round; r < kLogRounds; ++r) a.log.leaf[((size_t)chunk * kLogRounds + r) * 32 + lane] = kEmpty;
   if (!hit) return;
+  if (kShade == kShadePick) {
+    __stcs(a.out.nseg + i, acc.nseg);
+    return;
+  }
   if (kShade != kShadeAlpha) {
 #pragma unroll
     for (int ch = 0; ch < 3; ++ch) __stcs(a.out.rgb + 3 * i + ch, acc.C[ch]);
@@ -193,11 +201,15 @@ __device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, i
 // warp takes the next 32-ray packet from the counter when it finishes one, so
 // a long ray holds up only its own warp, not the other warps of its block.
 template <int KP, int DEG, typename E, int kShade = kShadeTree>
-__global__ void __launch_bounds__(256, packet_min_blocks<KP, DEG, E>()) render_packet_kernel(const __grid_constant__ FwdArgs a, int ready) {
+__global__ void __launch_bounds__(256, density_only(kShade) ? 4 : packet_min_blocks<KP, DEG, E>())
+    render_packet_kernel(const __grid_constant__ FwdArgs a, int ready) {
   // one packet per warp of the grid, or (with a work counter) packets pulled
   // one after another until the counter passes the last
   const int lane = threadIdx.x & 31;
-  const long long n_packets = (a.rays.n + 31) >> 5;
+  const long long n_live = a.n_live ? (long long)__ldg(a.n_live) : a.rays.n;
+  const uint32_t n_first = a.list ? __ldg(a.counts) : 0u;
+  const long long n_packets = (n_live + 31) >> 5;
+  const long long n_parts = a.list ? (long long)n_first + __ldg(a.counts + 1) : n_packets << a.split;
   if (a.log.n_chunks && blockIdx.x == 0 && threadIdx.x == 0) {
     a.log.header[0] = a.log.n_chunks;
     a.log.header[1] = kLogRounds;
@@ -205,22 +217,211 @@ __global__ void __launch_bounds__(256, packet_min_blocks<KP, DEG, E>()) render_p
     a.log.header[3] = (uint32_t)(a.rays.n >> 32);
     a.log.header[4] = 1u;
     a.log.header[5] = a.perm ? 1u : 0u;
+    if (!a.n_live) {
+      a.log.header[6] = (uint32_t)(n_live & 0xFFFFFFFFll);
+      a.log.header[7] = (uint32_t)(n_live >> 32);
+    }
   }
-  long long pk = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  long long k = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (a.work) {
     unsigned long long q = 0;
     if (lane == 0) q = atomicAdd(a.work, 1ull);
-    pk = (long long)__shfl_sync(0xFFFFFFFFu, q, 0);
+    k = (long long)__shfl_sync(kFull, q, 0);
   }
-  while (pk < n_packets) {
-    if (a.order) pk = (long long)min(__ldg(a.order + pk), (uint32_t)(n_packets - 1));
-    packet_forward<KP, DEG, E, kShade>(a, pk, ready);
+  while (k < n_parts) {
+    long long pk = k >> a.split;
+    int split = a.split, part = (int)(k & ((1 << a.split) - 1));
+    if (a.order) {
+      pk = (long long)min(__ldg(a.order + k), (uint32_t)(n_packets - 1));
+    } else if (a.list) {
+      const uint32_t v = __ldg(a.list + (k < n_first ? k : kQueueEntries - 1 - (k - n_first)));
+      pk = v & 0xFFFFFu;
+      split = (int)(v >> 20) & 3;
+      part = (int)(v >> 24);
+    }
+    packet_forward<KP, DEG, E, kShade>(a, pk, split, part, n_live, ready);
     __syncwarp();
     if (!a.work) break;
     unsigned long long q = 0;
     if (lane == 0) q = atomicAdd(a.work, 1ull);
-    pk = (long long)__shfl_sync(0xFFFFFFFFu, q, 0);
+    k = (long long)__shfl_sync(kFull, q, 0);
   }
+}
+
+// ---------------------------------------------------------------------------
+// Triage of a forward call of more packets than warps are resident.  Most
+// rays of a view miss the tree (72 % of the 8-view step's), and a packet
+// that missed cost the packet kernel a trip to the work counter and to its
+// rays; and a single long packet taken late kept a few SMs busy after the
+// others had finished (SMs active for 77 % of a 1080p view's time).
+// ---------------------------------------------------------------------------
+
+// Packets as given: writes the outputs of packets whose rays all miss the
+// box and lists the parts the others are run in.  A packet's work is estimated
+// from one point of each of its rays (a different fraction of the way through
+// the box for each lane): the brick-map cells that hold something, per ray, as
+// 32 such points see them.  Packets of `quarter` or more are run in four
+// parts, from `half` in two, these at the front of list (counts[0]) and so
+// first; the others whole, from its end backwards (counts[1]).
+__global__ void __launch_bounds__(256) triage_packets_kernel(const __grid_constant__ DevTree tr, const DevRays rays,
+                                                             const DevOut out, float half, float quarter,
+                                                             uint32_t *list, uint32_t *counts) {
+  __shared__ int parts[8];  // parts of each of the block's packets (0: none)
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  bool hit = false;
+  float cells = 0.f;
+  if (i < rays.n) {
+    float o[3], d[3], t, s_in, s_out;
+    load_ray(rays, i, o, d, t);
+    hit = ray_meets_box(tr, o, d, s_in, s_out);
+    if (hit) {
+      // bit-reversed lane: neighbouring rays look at distant depths
+      const float s = fmaf(((float)(__brev((unsigned)lane) >> 27) + 0.5f) * (1.f / 32.f), s_out - s_in, s_in);
+      const int Lc = tr.brick_level, mask = (1 << tr.depth) - 1;
+      uint32_t idx = 0u;
+      float len2 = 0.f;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const float g = (fmaf(s, d[a], o[a]) - tr.bmin[a]) * tr.scale[a], e = (s_out - s_in) * d[a] * tr.scale[a];
+        idx = (idx << Lc) | (uint32_t)(min(max((int)g, 0), mask) >> kBrickShift);
+        len2 = fmaf(e, e, len2);
+      }
+      if ((__ldg(tr.coarse + idx) >> 28) != kCoarseEmpty) cells = sqrtf(len2) * (1.f / (32 << kBrickShift));
+    }
+  }
+  const unsigned hits = __ballot_sync(kFull, hit);
+  if (!hits && i < rays.n) write_miss(out, i);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) cells += __shfl_xor_sync(kFull, cells, o);
+  if (lane == 0) parts[wid] = !hits ? 0 : (cells >= quarter ? 4 : (cells >= half ? 2 : 1));
+  __syncthreads();
+  if (wid == 0) {
+    // the block's packets in order, one add per count and block
+    const int p = lane < 8 ? parts[lane] : 0;
+    int incl = p > 1 ? p : 0;
+    const unsigned whole = __ballot_sync(kFull, p == 1);
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+      const int y = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += y;
+    }
+    const int total = __shfl_sync(kFull, incl, 7);
+    uint32_t bf = 0u, bl = 0u;
+    if (lane == 0) {
+      if (total) bf = atomicAdd(counts, (uint32_t)total);
+      if (whole) bl = atomicAdd(counts + 1, (uint32_t)__popc(whole));
+    }
+    bf = __shfl_sync(kFull, bf, 0) + (uint32_t)incl - (uint32_t)p;
+    bl = __shfl_sync(kFull, bl, 0) + (uint32_t)__popc(whole & ((1u << lane) - 1u));
+    const uint32_t pk = blockIdx.x * 8 + lane;
+    if (p == 1) list[kQueueEntries - 1 - bl] = part_entry(pk, 0, 0);
+    for (int k = 0; k < p && p > 1; ++k) list[bf + k] = part_entry(pk, p == 4 ? 2 : 1, k);
+  }
+}
+
+// Calls with a segment log (whose permutation the adjoint follows): packets
+// are formed from the rays that meet the box, block by block in the given
+// order, perm[0 .. *n_live); the others' outputs are written here and they
+// fill perm from its end.
+constexpr int kTriageBlock = 1024;
+__global__ void __launch_bounds__(kTriageBlock) triage_rays_kernel(const __grid_constant__ DevTree tr, const DevRays rays,
+                                                                   const DevOut out, uint32_t *perm, uint32_t *n_live,
+                                                                   uint32_t *n_miss) {
+  __shared__ uint32_t sum[kTriageBlock / 32], base_hit, base_miss;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool in = i < rays.n;
+  bool hit = false;
+  if (in) {
+    float o[3], d[3], t;
+    load_ray(rays, i, o, d, t);
+    float s_in, s_out;
+    hit = ray_meets_box(tr, o, d, s_in, s_out);
+    if (!hit) write_miss(out, i);
+  }
+  const unsigned hits = __ballot_sync(kFull, hit);
+  if (lane == 0) sum[wid] = (uint32_t)__popc(hits);
+  __syncthreads();
+  if (wid == 0) {
+    const uint32_t own = sum[lane];
+    uint32_t incl = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += y;
+    }
+    sum[lane] = incl - own;
+    if (lane == 31) {
+      const uint32_t rays_here = (uint32_t)min(rays.n - (long long)blockIdx.x * blockDim.x, (long long)kTriageBlock);
+      base_hit = incl ? atomicAdd(n_live, incl) : 0u;
+      base_miss = rays_here > incl ? atomicAdd(n_miss, rays_here - incl) : 0u;
+    }
+  }
+  __syncthreads();
+  if (!in) return;
+  const uint32_t before = sum[wid] + (uint32_t)__popc(hits & ((1u << lane) - 1u));  // hits before this ray in the block
+  if (hit) perm[base_hit + before] = (uint32_t)i;
+  else perm[rays.n - 1 - (base_miss + (threadIdx.x - before))] = (uint32_t)i;
+}
+
+// Bricks per ray, per packet of a resident warp's share, from which a packet
+// counts as long (see packet_launch).
+constexpr float kLongShare = 0.4f;
+
+// Launches a packet forward of any shading.  Up to four packets per resident
+// warp: a plain grid without counter or triage, each packet in as many parts
+// (up to four) as keep to that number, since these calls are bound by the
+// latency of their longest packet (without a log, whose layout is by whole
+// packets).  Above: a persistent grid on the work counter, after the triage
+// that the call allows: of rays with a log in which the packets are taken as
+// given (n < 2^32), of packets without a log on trees with a brick map.
+template <int KP, int DEG, typename E, int kShade>
+static cudaError_t packet_launch(FwdArgs a, const LaunchCfg &cfg, cudaStream_t s) {
+  if (a.rays.n == 0) return cudaSuccess;
+  const long long n_packets = (a.rays.n + 31) >> 5;
+  const int warps = cfg.block / 32;
+  const size_t sm = smem_bytes(cfg.block, KP, shade_chunks<KP, DEG, E, kShade>(), path_words(a.tr));
+  cudaError_t e;
+  if (sm > 48 * 1024 && (e = cudaFuncSetAttribute(render_packet_kernel<KP, DEG, E, kShade>,
+                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
+    return e;
+  int per_sm = 0;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, render_packet_kernel<KP, DEG, E, kShade>, cfg.block,
+                                                         sm)) != cudaSuccess)
+    return e;
+  const long long want = (long long)(per_sm > 0 ? per_sm : 1) * cfg.num_sms;  // resident blocks
+  const long long resident = want * warps;
+  if (!a.log.n_chunks)
+    while (a.split < kMaxSplit && (n_packets << (a.split + 1)) <= 4 * resident) ++a.split;
+  long long grid = ((n_packets << a.split) + warps - 1) / warps;
+  if (grid <= want || a.split) a.work = nullptr;
+  if (a.work) {
+    grid = want;
+    if ((e = cudaMemsetAsync(a.work, 0, 2 * sizeof(unsigned long long), s)) != cudaSuccess) return e;
+    if (a.log.n_chunks && !a.order && !a.perm && a.rays.n <= 0xFFFFFFFFll) {
+      uint32_t *live = a.log.header + 6;
+      if ((e = cudaMemsetAsync(a.log.heads, 0xFF, (size_t)((char *)(a.log.key + n_packets) - (char *)a.log.heads), s)) !=
+          cudaSuccess)
+        return e;
+      triage_rays_kernel<<<(unsigned)((a.rays.n + kTriageBlock - 1) / kTriageBlock), kTriageBlock, 0, s>>>(
+          a.tr, a.rays, a.out, a.log.perm, live, a.log.header + 8);
+      a.perm = a.log.perm;
+      a.n_live = live;
+    } else if (!a.log.n_chunks && a.queue && a.tr.coarse && n_packets <= kQueuePackets) {
+      // a packet is long when its work is a notable part of an average warp's
+      // share, which grows with the packets per resident warp
+      uint32_t *counts = reinterpret_cast<uint32_t *>(a.work + 1);
+      const float half = kLongShare * (float)n_packets / (float)resident;
+      triage_packets_kernel<<<(unsigned)((a.rays.n + 255) / 256), 256, 0, s>>>(a.tr, a.rays, a.out, half, 2.f * half,
+                                                                               a.queue, counts);
+      a.list = a.queue;
+      a.counts = counts;
+    }
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  render_packet_kernel<KP, DEG, E, kShade><<<(unsigned)grid, cfg.block, sm, s>>>(a, cfg.ready);
+  return cudaGetLastError();
 }
 
 __global__ void __launch_bounds__(256) trace_kernel(const __grid_constant__ TraceArgs a) {
@@ -253,31 +454,9 @@ __global__ void __launch_bounds__(256) trace_kernel(const __grid_constant__ Trac
 
 template <int KP, int DEG, typename E>
 static cudaError_t fwd_one(bool packet, const FwdArgs &a, const LaunchCfg &cfg, cudaStream_t s) {
+  if (packet) return packet_launch<KP, DEG, E, kShadeTree>(a, cfg, s);
   if (a.rays.n == 0) return cudaSuccess;
-  const long long blocks = (a.rays.n + cfg.block - 1) / cfg.block;
-  if (!packet) {
-    render_plain_kernel<KP, DEG, E><<<(unsigned)blocks, cfg.block, 0, s>>>(a);
-  } else {
-    const size_t sm = smem_bytes(cfg.block, KP, shade_chunks<KP, DEG, E, kShadeTree>(), path_words(a.tr));
-    if (sm > 48 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(render_packet_kernel<KP, DEG, E>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-      if (e != cudaSuccess) return e;
-    }
-    if (!a.work) {
-      render_packet_kernel<KP, DEG, E><<<(unsigned)blocks, cfg.block, sm, s>>>(a, cfg.ready);
-    } else {
-      int per_sm = 0;
-      cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, render_packet_kernel<KP, DEG, E>,
-                                                                    cfg.block, sm);
-      if (e != cudaSuccess) return e;
-      const long long want = (long long)(per_sm > 0 ? per_sm : 1) * cfg.num_sms;
-      e = cudaMemsetAsync(a.work, 0, sizeof(unsigned long long), s);
-      if (e != cudaSuccess) return e;
-      render_packet_kernel<KP, DEG, E><<<(unsigned)(want < blocks ? want : blocks), cfg.block, sm, s>>>(
-          a, cfg.ready);
-    }
-  }
+  render_plain_kernel<KP, DEG, E><<<(unsigned)((a.rays.n + cfg.block - 1) / cfg.block), cfg.block, 0, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -503,26 +682,7 @@ cudaError_t launch_slice(int KP, int DEG, DType dt, const DevTree &tr, float u, 
 // the storage type only sets the register budget, 128 per thread).
 template <int DEG>
 static cudaError_t render_slice_one(const FwdArgs &a, const LaunchCfg &cfg, cudaStream_t s) {
-  if (a.rays.n == 0) return cudaSuccess;
-  const long long blocks = (a.rays.n + cfg.block - 1) / cfg.block;
-  const bool persistent = a.work != nullptr;
-  cudaError_t e;
-  if (persistent && (e = cudaMemsetAsync(a.work, 0, sizeof(unsigned long long), s)) != cudaSuccess) return e;
-  const size_t sm = smem_bytes(cfg.block, 8, shade_chunks<8, DEG, __nv_bfloat16, kShadeSlice>(), path_words(a.tr));
-  if (sm > 48 * 1024 && (e = cudaFuncSetAttribute(render_packet_kernel<8, DEG, __nv_bfloat16, kShadeSlice>,
-                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
-    return e;
-  long long grid = blocks;
-  if (persistent) {
-    int per_sm = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, render_packet_kernel<8, DEG, __nv_bfloat16, kShadeSlice>,
-                                                           cfg.block, sm)) != cudaSuccess)
-      return e;
-    const long long want = (long long)(per_sm > 0 ? per_sm : 1) * cfg.num_sms;
-    if (want < grid) grid = want;
-  }
-  render_packet_kernel<8, DEG, __nv_bfloat16, kShadeSlice><<<(unsigned)grid, cfg.block, sm, s>>>(a, cfg.ready);
-  return cudaGetLastError();
+  return packet_launch<8, DEG, __nv_bfloat16, kShadeSlice>(a, cfg, s);
 }
 
 cudaError_t launch_render_slice(int DEG, const FwdArgs &a, const LaunchCfg &cfg, cudaStream_t s) {
@@ -534,61 +694,35 @@ cudaError_t launch_render_slice(int DEG, const FwdArgs &a, const LaunchCfg &cfg,
 
 // Terminating voxel of each ray (Sec. 5 "Appearance editing"): the leaf of the
 // segment at which 1 - exp(-sum sigma delta) of the unedited render first
-// reaches the threshold; -1 when it never does.  One thread per ray.
+// reaches the threshold; -1 when it never does.  The density-only packet
+// forward with the threshold in the place of the early stop.
 template <int KP, int DEG, typename E>
-__global__ void __launch_bounds__(256) pick_kernel(const __grid_constant__ FwdArgs a, float threshold, int *leaf_out) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= a.rays.n) return;
-  float o[3], d[3], t, dn[3];
-  load_ray(a.rays, i, o, d, t);
-  int picked = -1;
-  RayWalk w;
-  if (walk_init(a.tr, o, d, w, dn)) {
-    RayConst<KP, DEG> rc;
-    ray_const_basis<KP, DEG>(a.tr, t * (float)(a.tr.T - 1), rc);
-    const RegRows<KP> rows{rc.a, rc.b};
-    float optical = 0.f;
-    uint32_t leaf;
-    float t0, dt;
-    while (walk_next(a.tr, w, leaf, t0, dt)) {
-      LeafRecord<KP, DEG, E> rec;
-      rec.load_sigma(a.tr, leaf);
-      optical = fmaf(fmaxf(pre_sigma_of<KP>(rows, rec), 0.f), dt, optical);
-      if (-expm1f(-optical) >= threshold) {
-        picked = (int)leaf;
-        break;
-      }
-    }
-  }
-  leaf_out[i] = picked;
+static cudaError_t pick_one(FwdArgs a, float threshold, int *leaf_out, const LaunchCfg &cfg, cudaStream_t s) {
+  a.t_stop = threshold;
+  a.out = DevOut{nullptr, nullptr, nullptr, nullptr, leaf_out};
+  return packet_launch<KP, DEG, E, kShadePick>(a, cfg, s);
 }
 
-template <int KP, int DEG, typename E>
-static cudaError_t pick_one(const FwdArgs &a, float threshold, int *leaf_out, cudaStream_t s) {
-  if (a.rays.n == 0) return cudaSuccess;
-  pick_kernel<KP, DEG, E><<<(unsigned)((a.rays.n + 127) / 128), 128, 0, s>>>(a, threshold, leaf_out);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_pick(int KP, int DEG, DType dt, const FwdArgs &a, float threshold, int *leaf_out, cudaStream_t s) {
+cudaError_t launch_pick(int KP, int DEG, DType dt, const FwdArgs &a, float threshold, int *leaf_out,
+                        const LaunchCfg &cfg, cudaStream_t s) {
 #define NEUVV_PICK_KD(E)                                   \
   switch (KP * 10 + DEG) {                                 \
-    case 81: return pick_one<8, 1, E>(a, threshold, leaf_out, s);   \
-    case 82: return pick_one<8, 2, E>(a, threshold, leaf_out, s);   \
-    case 83: return pick_one<8, 3, E>(a, threshold, leaf_out, s);   \
-    case 161: return pick_one<16, 1, E>(a, threshold, leaf_out, s); \
-    case 162: return pick_one<16, 2, E>(a, threshold, leaf_out, s); \
-    case 163: return pick_one<16, 3, E>(a, threshold, leaf_out, s); \
-    case 321: return pick_one<32, 1, E>(a, threshold, leaf_out, s); \
-    case 322: return pick_one<32, 2, E>(a, threshold, leaf_out, s); \
-    case 323: return pick_one<32, 3, E>(a, threshold, leaf_out, s); \
+    case 81: return pick_one<8, 1, E>(a, threshold, leaf_out, cfg, s);   \
+    case 82: return pick_one<8, 2, E>(a, threshold, leaf_out, cfg, s);   \
+    case 83: return pick_one<8, 3, E>(a, threshold, leaf_out, cfg, s);   \
+    case 161: return pick_one<16, 1, E>(a, threshold, leaf_out, cfg, s); \
+    case 162: return pick_one<16, 2, E>(a, threshold, leaf_out, cfg, s); \
+    case 163: return pick_one<16, 3, E>(a, threshold, leaf_out, cfg, s); \
+    case 321: return pick_one<32, 1, E>(a, threshold, leaf_out, cfg, s); \
+    case 322: return pick_one<32, 2, E>(a, threshold, leaf_out, cfg, s); \
+    case 323: return pick_one<32, 3, E>(a, threshold, leaf_out, cfg, s); \
     default: return cudaErrorInvalidValue;                 \
   }
   if (dt == kF32) NEUVV_PICK_KD(float)
   if (dt == kBF16) NEUVV_PICK_KD(__nv_bfloat16)
 #undef NEUVV_PICK_KD
-  if (KP == 8 && DEG == 2) return pick_one<8, 2, Fp8E4M3>(a, threshold, leaf_out, s);
-  if (KP == 16 && DEG == 3) return pick_one<16, 3, Fp8E4M3>(a, threshold, leaf_out, s);
+  if (KP == 8 && DEG == 2) return pick_one<8, 2, Fp8E4M3>(a, threshold, leaf_out, cfg, s);
+  if (KP == 16 && DEG == 3) return pick_one<16, 3, Fp8E4M3>(a, threshold, leaf_out, cfg, s);
   return cudaErrorInvalidValue;
 }
 
@@ -627,71 +761,34 @@ cudaError_t launch_paint(const int *leaf, const float *color, long long n, long 
   return cudaGetLastError();
 }
 
-// Packet render with appearance edits (built for the two record shapes of the
-// workloads: K_pad 8 with degree 2, K_pad 16 with degree 3).
-template <int KP, int DEG, typename E>
-static cudaError_t edit_one(const FwdArgs &a, const LaunchCfg &cfg, cudaStream_t s) {
-  if (a.rays.n == 0) return cudaSuccess;
-  const long long blocks = (a.rays.n + cfg.block - 1) / cfg.block;
-  const size_t sm = smem_bytes(cfg.block, KP, shade_chunks<KP, DEG, E, kShadeEdit>(), path_words(a.tr));
-  cudaError_t e;
-  if (sm > 48 * 1024 && (e = cudaFuncSetAttribute(render_packet_kernel<KP, DEG, E, kShadeEdit>,
-                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
-    return e;
-  long long grid = blocks;
-  if (a.work) {
-    int per_sm = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, render_packet_kernel<KP, DEG, E, kShadeEdit>,
-                                                           cfg.block, sm)) != cudaSuccess)
-      return e;
-    const long long want = (long long)(per_sm > 0 ? per_sm : 1) * cfg.num_sms;
-    if (want < grid) grid = want;
-    if ((e = cudaMemsetAsync(a.work, 0, sizeof(unsigned long long), s)) != cudaSuccess) return e;
-  }
-  render_packet_kernel<KP, DEG, E, kShadeEdit><<<(unsigned)grid, cfg.block, sm, s>>>(a, cfg.ready);
-  return cudaGetLastError();
-}
-
 // Density-only packet render (alpha, depth, tau and nseg of the full render,
 // no colour): one packet per warp of a full grid, no work counter, so it may
 // run beside other calls on the same tree.  Built for the two record shapes
-// of the workloads (K_pad 8 with degree 2, K_pad 16 with degree 3).
-template <int KP, int DEG, typename E>
-static cudaError_t alpha_one(const FwdArgs &a, const LaunchCfg &cfg, cudaStream_t s) {
-  if (a.rays.n == 0) return cudaSuccess;
-  const long long blocks = (a.rays.n + cfg.block - 1) / cfg.block;
-  const size_t sm = smem_bytes(cfg.block, KP, shade_chunks<KP, DEG, E, kShadeAlpha>(), path_words(a.tr));
-  cudaError_t e;
-  if (sm > 48 * 1024 && (e = cudaFuncSetAttribute(render_packet_kernel<KP, DEG, E, kShadeAlpha>,
-                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
-    return e;
-  render_packet_kernel<KP, DEG, E, kShadeAlpha><<<(unsigned)blocks, cfg.block, sm, s>>>(a, cfg.ready);
-  return cudaGetLastError();
-}
-
+// of the workloads (K_pad 8 with degree 2, K_pad 16 with degree 3), as are
+// the renders with appearance edits.
 cudaError_t launch_render_alpha(int KP, int DEG, DType dt, const FwdArgs &a, const LaunchCfg &cfg, cudaStream_t s) {
   if (a.work || a.log.n_chunks) return cudaErrorInvalidValue;
   if (KP == 8 && DEG == 2) {
-    if (dt == kF32) return alpha_one<8, 2, float>(a, cfg, s);
-    if (dt == kBF16) return alpha_one<8, 2, __nv_bfloat16>(a, cfg, s);
-    return alpha_one<8, 2, Fp8E4M3>(a, cfg, s);
+    if (dt == kF32) return packet_launch<8, 2, float, kShadeAlpha>(a, cfg, s);
+    if (dt == kBF16) return packet_launch<8, 2, __nv_bfloat16, kShadeAlpha>(a, cfg, s);
+    return packet_launch<8, 2, Fp8E4M3, kShadeAlpha>(a, cfg, s);
   }
   if (KP == 16 && DEG == 3) {
-    if (dt == kF32) return alpha_one<16, 3, float>(a, cfg, s);
-    if (dt == kBF16) return alpha_one<16, 3, __nv_bfloat16>(a, cfg, s);
-    return alpha_one<16, 3, Fp8E4M3>(a, cfg, s);
+    if (dt == kF32) return packet_launch<16, 3, float, kShadeAlpha>(a, cfg, s);
+    if (dt == kBF16) return packet_launch<16, 3, __nv_bfloat16, kShadeAlpha>(a, cfg, s);
+    return packet_launch<16, 3, Fp8E4M3, kShadeAlpha>(a, cfg, s);
   }
   return cudaErrorNotSupported;
 }
 
 cudaError_t launch_render_edit(int KP, int DEG, DType dt, const FwdArgs &a, const LaunchCfg &cfg, cudaStream_t s) {
   if (KP == 8 && DEG == 2) {
-    if (dt == kF32) return edit_one<8, 2, float>(a, cfg, s);
-    if (dt == kBF16) return edit_one<8, 2, __nv_bfloat16>(a, cfg, s);
+    if (dt == kF32) return packet_launch<8, 2, float, kShadeEdit>(a, cfg, s);
+    if (dt == kBF16) return packet_launch<8, 2, __nv_bfloat16, kShadeEdit>(a, cfg, s);
   }
   if (KP == 16 && DEG == 3) {
-    if (dt == kF32) return edit_one<16, 3, float>(a, cfg, s);
-    if (dt == kBF16) return edit_one<16, 3, __nv_bfloat16>(a, cfg, s);
+    if (dt == kF32) return packet_launch<16, 3, float, kShadeEdit>(a, cfg, s);
+    if (dt == kBF16) return packet_launch<16, 3, __nv_bfloat16, kShadeEdit>(a, cfg, s);
   }
   return cudaErrorNotSupported;
 }
