@@ -828,9 +828,11 @@ neuvv_status neuvv_render(const neuvv_tree *t, const neuvv_rays *rays, float tim
     } else if (cfg.order == 2 && (size_t)chunk_bytes >= ray_order_scratch_bytes(rays->n)) {
       // packets re-formed from the rays sorted by direction and region (the
       // chunk area is the sort's scratch until the forward writes it)
-      if ((e = launch_ray_order(a.tr, a.rays, a.log.perm, a.log.next, cfg.num_sms, st)) != cudaSuccess)
+      if ((e = launch_ray_order(a.tr, a.rays, a.out, a.log.perm, a.log.header + 6, a.log.header + 8, a.log.next,
+                                cfg.num_sms, st)) != cudaSuccess)
         return cuda_fail(e, "ray order");
       a.perm = a.log.perm;
+      a.n_live = a.log.header + 6;
     }
   } else if ((e = clear_log(out, st)) != cudaSuccess) {
     return cuda_fail(e, "clear log");

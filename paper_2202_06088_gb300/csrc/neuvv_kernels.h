@@ -215,8 +215,13 @@ cudaError_t launch_exclusive_scan(uint32_t *v, long long n, uint32_t *part, int 
 // by (direction bucket, region of the first leaf), stable; scratch of
 // ray_order_scratch_bytes(n) bytes.
 size_t ray_order_scratch_bytes(long long n);
-cudaError_t launch_ray_order(const DevTree &tr, const DevRays &rays, uint32_t *perm, void *scratch, int num_sms,
-                             cudaStream_t s);
+cudaError_t launch_ray_order(const DevTree &tr, const DevRays &rays, const DevOut &out, uint32_t *perm,
+                             uint32_t *n_live, uint32_t *n_miss, void *scratch, int num_sms, cudaStream_t s);
+// Lists the rays that meet the tree's box in hits[0 .. *n_live) (n < 2^32),
+// writes the outputs of the others and lists them from the end of misses,
+// backwards (*n_miss; both counters zero before).
+cudaError_t launch_triage_rays(const DevTree &tr, const DevRays &rays, const DevOut &out, uint32_t *hits,
+                               uint32_t *misses, uint32_t *n_live, uint32_t *n_miss, cudaStream_t s);
 // Packets in region order for the forward (cfg.order == 1): each packet's key
 // is the first leaf that its first hitting ray (of lanes 0, 8, 16, 24)
 // reaches (leaf ids follow the Morton order of the leaves), counting-sorted

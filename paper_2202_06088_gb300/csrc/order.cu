@@ -8,7 +8,9 @@
 // of the leaf id, which follows the Morton order of the leaves) in the low
 // 18 -- and a stable LSD radix sort (three passes of 8-bit digits) lists the
 // rays by key.  Rays of one view that enter one region of the tree become
-// neighbours; rays with equal keys keep the caller's order.  The result is a
+// neighbours; rays with equal keys keep the order of the list they are sorted
+// from, the rays that meet the tree's box (the caller's order, block by block).
+// Rays that miss it come last, unsorted.  The result is a
 // permutation (position -> ray) that the packet forward and adjoint read
 // their rays through; outputs stay in the caller's order.
 #include <algorithm>
@@ -131,10 +133,15 @@ __device__ __forceinline__ uint32_t direction_bucket(const float d[3]) {
   return (uint32_t)(u * 8 + v);
 }
 
+// Keys of the listed rays (those that meet the tree's box: of a batch drawn
+// over whole views, where three in four miss, a thread per ray of the batch
+// walked with a quarter of its lanes).
 __global__ void __launch_bounds__(256) ray_key_kernel(const __grid_constant__ DevTree tr, const DevRays rays,
-                                                      uint32_t *keys, uint32_t *perm, int shift) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= rays.n) return;
+                                                      const uint32_t *list, const uint32_t *n_list, uint32_t *keys,
+                                                      int shift) {
+  const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= (long long)__ldg(n_list)) return;
+  const long long i = __ldg(list + k);
   float o[3], d[3], t, dn[3];
   load_ray(rays, i, o, d, t);
   RayWalk w;
@@ -142,8 +149,7 @@ __global__ void __launch_bounds__(256) ray_key_kernel(const __grid_constant__ De
   float t0, dt;
   if (walk_init(tr, o, d, w, dn) && walk_next(tr, w, leaf, t0, dt))
     key = (direction_bucket(dn) << 18) | ((leaf >> shift) & 0x3FFFFu);
-  keys[i] = key;
-  perm[i] = (uint32_t)i;
+  keys[k] = key;
 }
 
 // ---------------------------------------------------------------------------
@@ -155,9 +161,10 @@ constexpr int kRadixWarps = 8, kRadixPerWarp = 512, kRadixTile = kRadixWarps * k
 constexpr int kRadixSteps = kRadixPerWarp / 32;
 
 // table[d * n_tiles + tile] = pairs of the tile with digit d.
-__global__ void __launch_bounds__(kRadixWarps * 32) radix_hist_kernel(const uint32_t *keys, long long n, int sh,
+__global__ void __launch_bounds__(kRadixWarps * 32) radix_hist_kernel(const uint32_t *keys, const uint32_t *n_keys, int sh,
                                                                        uint32_t *table, int n_tiles) {
   __shared__ uint32_t cnt[256];
+  const long long n = __ldg(n_keys);
   cnt[threadIdx.x] = 0;
   __syncthreads();
   const long long first = (long long)blockIdx.x * kRadixTile;
@@ -176,8 +183,10 @@ __global__ void __launch_bounds__(kRadixWarps * 32) radix_hist_kernel(const uint
 // keep their order.
 __global__ void __launch_bounds__(kRadixWarps * 32) radix_scatter_kernel(const uint32_t *keys_in, const uint32_t *perm_in,
                                                                           uint32_t *keys_out, uint32_t *perm_out,
-                                                                          long long n, int sh, const uint32_t *table,
-                                                                          int n_tiles) {
+                                                                          const uint32_t *n_keys, int sh,
+                                                                          const uint32_t *table, int n_tiles) {
+  const long long n = __ldg(n_keys);
+  if ((long long)blockIdx.x * kRadixTile >= n) return;
   __shared__ uint32_t wcnt[kRadixWarps][256];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int k = threadIdx.x; k < kRadixWarps * 256; k += blockDim.x) (&wcnt[0][0])[k] = 0;
@@ -225,8 +234,8 @@ size_t ray_order_scratch_bytes(long long n) {
   return (size_t)n * 16 + (size_t)(256 * tiles + 1) * 4 + (size_t)kScanParts * 4 + 256;
 }
 
-cudaError_t launch_ray_order(const DevTree &tr, const DevRays &rays, uint32_t *perm, void *scratch, int num_sms,
-                             cudaStream_t s) {
+cudaError_t launch_ray_order(const DevTree &tr, const DevRays &rays, const DevOut &out, uint32_t *perm,
+                             uint32_t *n_live, uint32_t *n_miss, void *scratch, int num_sms, cudaStream_t s) {
   const long long n = rays.n;
   if (n == 0) return cudaSuccess;
   const long long tiles = (n + kRadixTile - 1) / kRadixTile;
@@ -239,16 +248,18 @@ cudaError_t launch_ray_order(const DevTree &tr, const DevRays &rays, uint32_t *p
   int bits = 0;
   while (bits < 32 && ((long long)1 << bits) <= tr.n_leaves) ++bits;
   const int shift = bits > 18 ? bits - 18 : 0;
-  ray_key_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(tr, rays, ka, pa, shift);
-  cudaError_t e = cudaGetLastError();
+  // the rays that meet the box; the others are done, and end the permutation
+  cudaError_t e = launch_triage_rays(tr, rays, out, pa, perm, n_live, n_miss, s);
   if (e != cudaSuccess) return e;
+  ray_key_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(tr, rays, pa, n_live, ka, shift);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const uint32_t *kin = ka, *pin = pa;
   uint32_t *kout = kb, *pout = pb;
   for (int pass = 0; pass < 3; ++pass) {
     if (pass == 2) pout = perm;  // the last pass writes the permutation in place
-    radix_hist_kernel<<<(unsigned)tiles, kRadixWarps * 32, 0, s>>>(kin, n, 8 * pass, table, (int)tiles);
+    radix_hist_kernel<<<(unsigned)tiles, kRadixWarps * 32, 0, s>>>(kin, n_live, 8 * pass, table, (int)tiles);
     if ((e = launch_exclusive_scan(table, 256 * tiles, part, num_sms, s)) != cudaSuccess) return e;
-    radix_scatter_kernel<<<(unsigned)tiles, kRadixWarps * 32, 0, s>>>(kin, pin, kout, pout, n, 8 * pass, table,
+    radix_scatter_kernel<<<(unsigned)tiles, kRadixWarps * 32, 0, s>>>(kin, pin, kout, pout, n_live, 8 * pass, table,
                                                                       (int)tiles);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const uint32_t *tk = kout, *tp = pout;

@@ -321,12 +321,13 @@ __global__ void __launch_bounds__(256) triage_packets_kernel(const __grid_consta
 }
 
 // Calls with a segment log (whose permutation the adjoint follows): packets
-// are formed from the rays that meet the box, block by block in the given
-// order, perm[0 .. *n_live); the others' outputs are written here and they
-// fill perm from its end.
+// are formed from the rays that meet the box, listed block by block in the
+// given order; the others' outputs are written here and they are listed from
+// the end of miss_list.
 constexpr int kTriageBlock = 1024;
 __global__ void __launch_bounds__(kTriageBlock) triage_rays_kernel(const __grid_constant__ DevTree tr, const DevRays rays,
-                                                                   const DevOut out, uint32_t *perm, uint32_t *n_live,
+                                                                   const DevOut out, uint32_t *hit_list,
+                                                                   uint32_t *miss_list, uint32_t *n_live,
                                                                    uint32_t *n_miss) {
   __shared__ uint32_t sum[kTriageBlock / 32], base_hit, base_miss;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -361,8 +362,15 @@ __global__ void __launch_bounds__(kTriageBlock) triage_rays_kernel(const __grid_
   __syncthreads();
   if (!in) return;
   const uint32_t before = sum[wid] + (uint32_t)__popc(hits & ((1u << lane) - 1u));  // hits before this ray in the block
-  if (hit) perm[base_hit + before] = (uint32_t)i;
-  else perm[rays.n - 1 - (base_miss + (threadIdx.x - before))] = (uint32_t)i;
+  if (hit) hit_list[base_hit + before] = (uint32_t)i;
+  else miss_list[rays.n - 1 - (base_miss + (threadIdx.x - before))] = (uint32_t)i;
+}
+
+cudaError_t launch_triage_rays(const DevTree &tr, const DevRays &rays, const DevOut &out, uint32_t *hits,
+                               uint32_t *misses, uint32_t *n_live, uint32_t *n_miss, cudaStream_t s) {
+  triage_rays_kernel<<<(unsigned)((rays.n + kTriageBlock - 1) / kTriageBlock), kTriageBlock, 0, s>>>(
+      tr, rays, out, hits, misses, n_live, n_miss);
+  return cudaGetLastError();
 }
 
 // Bricks per ray, per packet of a resident warp's share, from which a packet
@@ -400,14 +408,11 @@ static cudaError_t packet_launch(FwdArgs a, const LaunchCfg &cfg, cudaStream_t s
     grid = want;
     if ((e = cudaMemsetAsync(a.work, 0, 2 * sizeof(unsigned long long), s)) != cudaSuccess) return e;
     if (a.log.n_chunks && !a.order && !a.perm && a.rays.n <= 0xFFFFFFFFll) {
-      uint32_t *live = a.log.header + 6;
-      if ((e = cudaMemsetAsync(a.log.heads, 0xFF, (size_t)((char *)(a.log.key + n_packets) - (char *)a.log.heads), s)) !=
+      a.perm = a.log.perm;
+      a.n_live = a.log.header + 6;
+      if ((e = launch_triage_rays(a.tr, a.rays, a.out, a.log.perm, a.log.perm, a.log.header + 6, a.log.header + 8, s)) !=
           cudaSuccess)
         return e;
-      triage_rays_kernel<<<(unsigned)((a.rays.n + kTriageBlock - 1) / kTriageBlock), kTriageBlock, 0, s>>>(
-          a.tr, a.rays, a.out, a.log.perm, live, a.log.header + 8);
-      a.perm = a.log.perm;
-      a.n_live = live;
     } else if (!a.log.n_chunks && a.queue && a.tr.coarse && n_packets <= kQueuePackets) {
       // a packet is long when its work is a notable part of an average warp's
       // share, which grows with the packets per resident warp
@@ -420,6 +425,10 @@ static cudaError_t packet_launch(FwdArgs a, const LaunchCfg &cfg, cudaStream_t s
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
+  // packets past the live rays are not run: no chunk, no key
+  if (a.n_live && (e = cudaMemsetAsync(a.log.heads, 0xFF, (size_t)((char *)(a.log.key + n_packets) - (char *)a.log.heads),
+                                       s)) != cudaSuccess)
+    return e;
   render_packet_kernel<KP, DEG, E, kShade><<<(unsigned)grid, cfg.block, sm, s>>>(a, cfg.ready);
   return cudaGetLastError();
 }
