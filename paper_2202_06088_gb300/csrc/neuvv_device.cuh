@@ -816,20 +816,33 @@ struct RayConst {
   float Y[(DEG + 1) * (DEG + 1)];
 };
 
+// Four consecutive values of the interpolated row of a basis table ([T][KP]
+// FP32, 16-byte aligned rows) between frames f0 and f1.
+__device__ __forceinline__ float4 basis_lerp4(const float *r0, const float *r1, int q, float fr) {
+  const float4 x = __ldg(reinterpret_cast<const float4 *>(r0) + q), y = __ldg(reinterpret_cast<const float4 *>(r1) + q);
+  return make_float4((1.f - fr) * x.x + fr * y.x, (1.f - fr) * x.y + fr * y.y, (1.f - fr) * x.z + fr * y.z,
+                     (1.f - fr) * x.w + fr * y.w);
+}
+// The two frames around frame coordinate u (clamped) and the weight of the second.
+__device__ __forceinline__ void basis_frames(const DevTree &tr, float u, int &f0, int &f1, float &fr) {
+  u = fminf(fmaxf(u, 0.f), (float)(tr.T - 1));
+  f0 = min((int)floorf(u), tr.T - 1);
+  f1 = min(f0 + 1, tr.T - 1);
+  fr = u - (float)f0;
+}
+
 // Frame coordinate u = t (T - 1) (t clamped to [0, 1]); rows lerped in u.
 template <int KP, int DEG>
 __device__ __forceinline__ void ray_const_basis(const DevTree &tr, float u, RayConst<KP, DEG> &rc) {
-  const float umax = (float)(tr.T - 1);
-  u = fminf(fmaxf(u, 0.f), umax);
-  int f0 = min((int)floorf(u), tr.T - 1);
-  const int f1 = min(f0 + 1, tr.T - 1);
-  const float fr = u - (float)f0;
-  const float *A0 = tr.A + (size_t)f0 * KP, *A1 = tr.A + (size_t)f1 * KP;
-  const float *B0 = tr.B + (size_t)f0 * KP, *B1 = tr.B + (size_t)f1 * KP;
+  int f0, f1;
+  float fr;
+  basis_frames(tr, u, f0, f1, fr);
 #pragma unroll
-  for (int k = 0; k < KP; ++k) {
-    rc.a[k] = (1.f - fr) * __ldg(A0 + k) + fr * __ldg(A1 + k);
-    rc.b[k] = (1.f - fr) * __ldg(B0 + k) + fr * __ldg(B1 + k);
+  for (int q = 0; q < KP / 4; ++q) {
+    const float4 a = basis_lerp4(tr.A + (size_t)f0 * KP, tr.A + (size_t)f1 * KP, q, fr);
+    const float4 b = basis_lerp4(tr.B + (size_t)f0 * KP, tr.B + (size_t)f1 * KP, q, fr);
+    rc.a[4 * q] = a.x, rc.a[4 * q + 1] = a.y, rc.a[4 * q + 2] = a.z, rc.a[4 * q + 3] = a.w;
+    rc.b[4 * q] = b.x, rc.b[4 * q + 1] = b.y, rc.b[4 * q + 2] = b.z, rc.b[4 * q + 3] = b.w;
   }
 }
 
@@ -873,49 +886,76 @@ struct Sample {
   float R[(DEG + 1) * (DEG + 2) / 2];
 };
 
-// Where a ray's interpolated basis rows a(u), b(u) live: registers
-// (RegRows) or a per-thread column of shared memory (SmemRows, entry k at
-// p[k * stride], b after a).
+// Where a ray's interpolated basis rows a(u), b(u) live, in quads: registers
+// (RegRows) or a column of shared memory (SmemRows: value k at p[k * stride], b
+// after a; lanes read the columns of any rays without bank conflicts, which
+// rows of quads at an odd pitch did not: 3.12 against 2.94 ms for the replay
+// of the 8-view step).
 template <int KP>
 struct RegRows {
   const float *a, *b;
-  __device__ __forceinline__ float A(int k) const { return a[k]; }
-  __device__ __forceinline__ float B(int k) const { return b[k]; }
+  __device__ __forceinline__ float4 A4(int q) const { return make_float4(a[4 * q], a[4 * q + 1], a[4 * q + 2], a[4 * q + 3]); }
+  __device__ __forceinline__ float4 B4(int q) const { return make_float4(b[4 * q], b[4 * q + 1], b[4 * q + 2], b[4 * q + 3]); }
 };
 template <int KP>
 struct SmemRows {
   const float *p;
   int stride;
-  __device__ __forceinline__ float A(int k) const { return p[k * stride]; }
-  __device__ __forceinline__ float B(int k) const { return p[(KP + k) * stride]; }
+  __device__ __forceinline__ float4 at(int k) const {
+    return make_float4(p[k * stride], p[(k + 1) * stride], p[(k + 2) * stride], p[(k + 3) * stride]);
+  }
+  __device__ __forceinline__ float4 A4(int q) const { return at(4 * q); }
+  __device__ __forceinline__ float4 B4(int q) const { return at(KP + 4 * q); }
 };
 
-// Frame coordinate u = t (T - 1), rows lerped in u, written to shared memory.
+// Rows at frame coordinate u written to shared memory (SmemRows).
 template <int KP>
 __device__ __forceinline__ void rows_to_smem(const DevTree &tr, float u, float *p, int stride) {
-  const float umax = (float)(tr.T - 1);
-  u = fminf(fmaxf(u, 0.f), umax);
-  const int f0 = min((int)floorf(u), tr.T - 1);
-  const int f1 = min(f0 + 1, tr.T - 1);
-  const float fr = u - (float)f0;
-  const float *A0 = tr.A + (size_t)f0 * KP, *A1 = tr.A + (size_t)f1 * KP;
-  const float *B0 = tr.B + (size_t)f0 * KP, *B1 = tr.B + (size_t)f1 * KP;
+  int f0, f1;
+  float fr;
+  basis_frames(tr, u, f0, f1, fr);
 #pragma unroll
-  for (int k = 0; k < KP; ++k) {
-    p[k * stride] = (1.f - fr) * __ldg(A0 + k) + fr * __ldg(A1 + k);
-    p[(KP + k) * stride] = (1.f - fr) * __ldg(B0 + k) + fr * __ldg(B1 + k);
+  for (int q = 0; q < KP / 4; ++q) {
+    const float4 a = basis_lerp4(tr.A + (size_t)f0 * KP, tr.A + (size_t)f1 * KP, q, fr);
+    const float4 b = basis_lerp4(tr.B + (size_t)f0 * KP, tr.B + (size_t)f1 * KP, q, fr);
+    float *pa = p + 4 * q * stride, *pb = pa + KP * stride;
+    pa[0] = a.x, pa[stride] = a.y, pa[2 * stride] = a.z, pa[3 * stride] = a.w;
+    pb[0] = b.x, pb[stride] = b.y, pb[2 * stride] = b.z, pb[3 * stride] = b.w;
   }
 }
+
+// sum_k row[k] w[k] as four partial sums (k mod 4), two to a packed FP32 FMA.
+__device__ __forceinline__ void ffma2(float &lo, float &hi, float a0, float a1, float b0, float b1) {
+  asm("{\n .reg .b64 a, b, c;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n mov.b64 c, {%0, %1};\n"
+      " fma.rn.f32x2 c, a, b, c;\n mov.b64 {%0, %1}, c;\n}"
+      : "+f"(lo), "+f"(hi)
+      : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
+}
+struct Dot4 {
+  float p[4] = {0.f, 0.f, 0.f, 0.f};
+  __device__ __forceinline__ void add(float4 r, float w0, float w1, float w2, float w3) {
+    ffma2(p[0], p[1], r.x, r.y, w0, w1);
+    ffma2(p[2], p[3], r.z, r.w, w2, w3);
+  }
+  __device__ __forceinline__ float sum() const { return (p[0] + p[1]) + (p[2] + p[3]); }
+};
 
 // Pre-activation density a(u) . w_sigma (Eq. project-sigma), four independent
 // FMA chains; the slice kernel forms it with the same operations.
 template <int KP, typename Rows, typename Rec>
 __device__ __forceinline__ float pre_sigma_of(const Rows &rows, const Rec &r) {
-  // four partial sums: independent FMA chains
-  float p4[4] = {0.f, 0.f, 0.f, 0.f};
+  Dot4 d;
 #pragma unroll
-  for (int k = 0; k < KP; ++k) p4[k & 3] = fmaf(rows.A(k), r.sig(k), p4[k & 3]);
-  return ((p4[0] + p4[1]) + (p4[2] + p4[3])) * r.scale_sigma();
+  for (int q = 0; q < KP / 4; ++q) d.add(rows.A4(q), r.sig(4 * q), r.sig(4 * q + 1), r.sig(4 * q + 2), r.sig(4 * q + 3));
+  return d.sum() * r.scale_sigma();
+}
+// Likewise b(u) . w_gamma (Eq. project-gamma).
+template <int KP, typename Rows, typename Rec>
+__device__ __forceinline__ float pre_gamma_of(const Rows &rows, const Rec &r) {
+  Dot4 d;
+#pragma unroll
+  for (int q = 0; q < KP / 4; ++q) d.add(rows.B4(q), r.gam(4 * q), r.gam(4 * q + 1), r.gam(4 * q + 2), r.gam(4 * q + 3));
+  return d.sum() * r.scale_gamma();
 }
 
 // Where a sample's record comes from: loaded before the evaluation (Loaded),
@@ -950,10 +990,7 @@ __device__ __forceinline__ void eval_sample(const DevTree &tr, const Rows &rows,
   s.sigma = fmaxf(ps, 0.f);
   if (!(s.sigma > 0.f)) return;
   src.template part<KP, 2 * KP>(r);
-  float q4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-  for (int k = 0; k < KP; ++k) q4[k & 3] = fmaf(rows.B(k), r.gam(k), q4[k & 3]);
-  const float pg = ((q4[0] + q4[1]) + (q4[2] + q4[3])) * r.scale_gamma();
+  const float pg = pre_gamma_of<KP>(rows, r);
   s.s_gamma = sigmoidf_fast(pg);
   sincospif(s.s_gamma, &s.sg, &s.cg);
   float dR[(DEG + 1) * (DEG + 2) / 2];

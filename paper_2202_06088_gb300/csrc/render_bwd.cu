@@ -127,10 +127,9 @@ __device__ __forceinline__ void scatter_gradient(const BwdArgs &a, const Rows &r
   }
 #pragma unroll
   for (int q = 0; q < KP / 4; ++q) {
-    red_add_v4(dst + 4 * q, dpre_s * rows.A(4 * q), dpre_s * rows.A(4 * q + 1), dpre_s * rows.A(4 * q + 2),
-               dpre_s * rows.A(4 * q + 3));
-    red_add_v4(dst + KP + 4 * q, dpre_g * rows.B(4 * q), dpre_g * rows.B(4 * q + 1), dpre_g * rows.B(4 * q + 2),
-               dpre_g * rows.B(4 * q + 3));
+    const float4 ra = rows.A4(q), rb = rows.B4(q);
+    red_add_v4(dst + 4 * q, dpre_s * ra.x, dpre_s * ra.y, dpre_s * ra.z, dpre_s * ra.w);
+    red_add_v4(dst + KP + 4 * q, dpre_g * rb.x, dpre_g * rb.y, dpre_g * rb.z, dpre_g * rb.w);
   }
   if (a.touched) {
     const unsigned int bit = 1u << (leaf & 31);
@@ -671,17 +670,14 @@ __device__ __forceinline__ void leaf_flush(const DevTree &tr, const LeafRecord<K
   RayConst<KP, DEG> rc;
   ray_const_basis<KP, DEG>(tr, u, rc);
   const RegRows<KP> rows{rc.a, rc.b};
-  float q4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-  for (int k = 0; k < KP; ++k) q4[k & 3] = fmaf(rows.B(k), rec.gam(k), q4[k & 3]);
-  const float pgam = ((q4[0] + q4[1]) + (q4[2] + q4[3])) * rec.scale_gamma();
+  const float pgam = pre_gamma_of<KP>(rows, rec);
   float sg, cg, R[(DEG + 1) * (DEG + 2) / 2];
   sincospif(sigmoidf_fast(pgam), &sg, &cg);
   hh_radial<DEG, false>(cg, sg, tr.hh_norm, R, nullptr);
 #pragma unroll
   for (int k = 0; k < KP; ++k) {
-    acc[k] = fmaf(ps, rows.A(k), acc[k]);
-    acc[KP + k] = fmaf(pg, rows.B(k), acc[KP + k]);
+    acc[k] = fmaf(ps, rc.a[k], acc[k]);
+    acc[KP + k] = fmaf(pg, rc.b[k], acc[KP + k]);
   }
   int j = 0;
 #pragma unroll

@@ -511,10 +511,7 @@ __device__ __forceinline__ void slice_row(const DevTree &tr, const RegRows<KP> &
 #pragma unroll
   for (int k = 0; k < NV * 4; ++k) out[k] = 0.f;
   out[0] = fmaxf(pre_sigma_of<KP>(rows, rec), 0.f);
-  float q4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-  for (int k = 0; k < KP; ++k) q4[k & 3] = fmaf(rows.B(k), rec.gam(k), q4[k & 3]);
-  const float pg = ((q4[0] + q4[1]) + (q4[2] + q4[3])) * rec.scale_gamma();
+  const float pg = pre_gamma_of<KP>(rows, rec);
   float sg, cg, R[(DEG + 1) * (DEG + 2) / 2];
   sincospif(sigmoidf_fast(pg), &sg, &cg);
   hh_radial<DEG, false>(cg, sg, tr.hh_norm, R, nullptr);
