@@ -120,46 +120,68 @@ __global__ void __launch_bounds__(kGradTileW *kGradTileH)
 
 
 // One warp per word of the touched bitmap (32 leaves): an empty word is
-// skipped at once, and each set bit's leaf is updated by the warp, one
-// 4-float quad of its record per lane, so a row is one coalesced access.
+// skipped at once.  A group of kGroup lanes takes a leaf, a lane a 4-float quad
+// of its record, so a row is one coalesced access (half a warp where 16 lanes
+// cover the record); each group loads two rows of gradient, master and moments
+// before it updates either.  DRAM bound: 4.8 of the measured 6.78 TB/s with
+// one row at a time by a whole warp (K_pad 8: 15 of 32 lanes at work).
+template <int kGroup>
 __global__ void __launch_bounds__(256) adam_kernel(float *__restrict__ master, float *__restrict__ m,
                                                    float *__restrict__ v, void *__restrict__ storage, int dt,
                                                    int storage_stride, float *__restrict__ grad,
                                                    const unsigned int *__restrict__ touched, long long n_leaves,
                                                    int stride_f32, int rec_len, float lr, float b1, float b2,
                                                    float eps, float c1, float c2) {
+  constexpr int kRows = 2;
   const int quads = (rec_len + 3) / 4;  // quads past the record's entries are padding and stay zero
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, group = lane / kGroup, q0 = lane % kGroup;
   const float lr_c1 = lr / c1, inv_c2 = 1.f / c2;
   const long long n_words = (n_leaves + 31) >> 5;
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
   for (long long wd = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; wd < n_words; wd += nwarps) {
     unsigned int bits = __ldg(touched + wd);  // the same for the whole warp
     while (bits) {
-      const long long leaf = (wd << 5) + (__ffs(bits) - 1);
-      bits &= bits - 1u;
-      for (int q = lane; q < quads; q += 32) {
-        const size_t off = (size_t)leaf * stride_f32 + 4 * q;
-        float4 g = *reinterpret_cast<const float4 *>(grad + off);
-        float4 w = *reinterpret_cast<const float4 *>(master + off);
-        float4 mm = *reinterpret_cast<const float4 *>(m + off);
-        float4 vv = *reinterpret_cast<const float4 *>(v + off);
-        float gs[4] = {g.x, g.y, g.z, g.w}, ws[4] = {w.x, w.y, w.z, w.w};
-        float ms[4] = {mm.x, mm.y, mm.z, mm.w}, vs[4] = {vv.x, vv.y, vv.z, vv.w};
+      // the next kRows * 32 / kGroup set bits, row r of group g the (r + kRows g)-th
+      long long leaf[kRows];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          if (4 * q + k >= rec_len) continue;  // padding stays zero
-          adam_entry(gs[k], b1, b2, lr_c1, inv_c2, eps, ws[k], ms[k], vs[k]);
+      for (int r = 0; r < kRows; ++r) leaf[r] = -1;
+#pragma unroll
+      for (int k = 0; k < kRows * 32 / kGroup; ++k) {
+        if (bits && k / kRows == group) leaf[k % kRows] = (wd << 5) + (__ffs(bits) - 1);
+        bits &= bits - 1u;  // 0 stays 0
+      }
+      for (int q = q0; q < quads; q += kGroup) {
+        float4 g[kRows], w[kRows], mm[kRows], vv[kRows];
+#pragma unroll
+        for (int r = 0; r < kRows; ++r) {
+          if (leaf[r] < 0) continue;
+          const size_t off = (size_t)leaf[r] * stride_f32 + 4 * q;
+          g[r] = *reinterpret_cast<const float4 *>(grad + off);
+          w[r] = *reinterpret_cast<const float4 *>(master + off);
+          mm[r] = *reinterpret_cast<const float4 *>(m + off);
+          vv[r] = *reinterpret_cast<const float4 *>(v + off);
         }
-        *reinterpret_cast<float4 *>(master + off) = make_float4(ws[0], ws[1], ws[2], ws[3]);
-        *reinterpret_cast<float4 *>(m + off) = make_float4(ms[0], ms[1], ms[2], ms[3]);
-        *reinterpret_cast<float4 *>(v + off) = make_float4(vs[0], vs[1], vs[2], vs[3]);
-        *reinterpret_cast<float4 *>(grad + off) = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (dt == kBF16) {
-          unsigned short *st = static_cast<unsigned short *>(storage) + (size_t)leaf * storage_stride + 4 * q;
-          const unsigned int lo = f32_to_bf16_rne(ws[0]) | ((unsigned int)f32_to_bf16_rne(ws[1]) << 16);
-          const unsigned int hi = f32_to_bf16_rne(ws[2]) | ((unsigned int)f32_to_bf16_rne(ws[3]) << 16);
-          *reinterpret_cast<uint2 *>(st) = make_uint2(lo, hi);
+#pragma unroll
+        for (int r = 0; r < kRows; ++r) {
+          if (leaf[r] < 0) continue;
+          const size_t off = (size_t)leaf[r] * stride_f32 + 4 * q;
+          float gs[4] = {g[r].x, g[r].y, g[r].z, g[r].w}, ws[4] = {w[r].x, w[r].y, w[r].z, w[r].w};
+          float ms[4] = {mm[r].x, mm[r].y, mm[r].z, mm[r].w}, vs[4] = {vv[r].x, vv[r].y, vv[r].z, vv[r].w};
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            if (4 * q + k >= rec_len) continue;  // padding stays zero
+            adam_entry(gs[k], b1, b2, lr_c1, inv_c2, eps, ws[k], ms[k], vs[k]);
+          }
+          *reinterpret_cast<float4 *>(master + off) = make_float4(ws[0], ws[1], ws[2], ws[3]);
+          *reinterpret_cast<float4 *>(m + off) = make_float4(ms[0], ms[1], ms[2], ms[3]);
+          *reinterpret_cast<float4 *>(v + off) = make_float4(vs[0], vs[1], vs[2], vs[3]);
+          *reinterpret_cast<float4 *>(grad + off) = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (dt == kBF16) {
+            unsigned short *st = static_cast<unsigned short *>(storage) + (size_t)leaf[r] * storage_stride + 4 * q;
+            const unsigned int lo = f32_to_bf16_rne(ws[0]) | ((unsigned int)f32_to_bf16_rne(ws[1]) << 16);
+            const unsigned int hi = f32_to_bf16_rne(ws[2]) | ((unsigned int)f32_to_bf16_rne(ws[3]) << 16);
+            *reinterpret_cast<uint2 *>(st) = make_uint2(lo, hi);
+          }
         }
       }
     }
@@ -331,8 +353,12 @@ cudaError_t launch_adam(float *master, float *m, float *v, void *storage, DType 
   }
   const long long want = ((n_leaves + 31) / 32 * 32 + 255) / 256;  // one warp per bitmap word
   const int blocks = (int)(want < 152 * 16 ? want : 152 * 16);
-  adam_kernel<<<blocks, 256, 0, s>>>(master, m, v, storage, (int)dt, storage_stride, grad, touched, n_leaves,
-                                     stride_f32, rec_len, lr, b1, b2, eps, c1, c2);
+  if (rec_len <= 64)
+    adam_kernel<16><<<blocks, 256, 0, s>>>(master, m, v, storage, (int)dt, storage_stride, grad, touched, n_leaves,
+                                           stride_f32, rec_len, lr, b1, b2, eps, c1, c2);
+  else
+    adam_kernel<32><<<blocks, 256, 0, s>>>(master, m, v, storage, (int)dt, storage_stride, grad, touched, n_leaves,
+                                           stride_f32, rec_len, lr, b1, b2, eps, c1, c2);
   return cudaGetLastError();
 }
 
