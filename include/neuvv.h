@@ -132,23 +132,26 @@ typedef struct {
   int64_t n_nodes, n_leaves;
   int32_t device;
   int32_t packet_block;     /* packet kernels: threads per block */
-  int32_t packet_queue;     /* packet kernels: leaf segments a ray may queue ahead of shading */
-  int32_t packet_ready;     /* packet kernels: lanes holding a queued segment that start a
-                               shading round (all three set by neuvv_autotune) */
+  int32_t packet_queue;     /* packet kernels: as set by the caller (a packet's segments wait in
+                               one ring, whose size is fixed) */
+  int32_t packet_ready;     /* packet kernels: waiting segments of a packet that start a shading
+                               batch (all three set by neuvv_autotune) */
   int32_t packet_order;     /* packet forward with a segment log: NEUVV_ORDER_* (neuvv_autotune) */
   int32_t packet_tiles;     /* pixel tile of a 32-ray packet of camera rays, NEUVV_TILES_*
                                (neuvv_autotune_tiles; default 8x4) */
 } neuvv_tree_info;
 
 /* The order in which the packet forward runs its 32-ray packets when the
- * call has a segment log (the rays themselves, their outputs and the packets'
- * contents do not change).  AS_GIVEN: in ray order.  BY_REGION: a pre-pass
+ * call has a segment log (the rays themselves and their outputs do not
+ * change).  AS_GIVEN: in ray order; when there are more packets than resident
+ * warps they are formed from the rays that meet the tree's box only, in that
+ * order by blocks of 1024 rays.  BY_REGION: a pre-pass
  * finds the first leaf each packet reaches and the packets run sorted by
  * that leaf's region (leaf ids follow the Morton order of the leaves), so
  * packets of different views that see the same part of the tree run
  * together and share its records in L2.  BY_RAY: the packets themselves are
- * re-formed: the rays are sorted (stable) by a bucket of their direction and
- * the region of the first leaf they reach, so a batch of rays from many
+ * re-formed: the rays that meet the box are sorted by a bucket of their
+ * direction and the region of the first leaf they reach, so a batch of rays from many
  * views and times in any order gets packets of rays that cross the same
  * cells; outputs stay in the caller's order, and the order is kept in the
  * log for the adjoint (it needs about 17 bytes per ray of the log as scratch,
@@ -169,7 +172,7 @@ typedef struct {
  * nseg: [n] segments composited (needed by the backward pass).  Any member may
  * be NULL except where a call says otherwise.
  * log, log_bytes: optional device buffer (16-byte aligned) in which the packet
- * forward records, per 32-ray packet, the leaf and chord of every segment it
+ * forward records, per 32-ray packet, the leaf, chord and ray of every segment it
  * composites, in shading order; neuvv_render_backward given the same saved
  * outputs replays a packet from the log instead of walking the tree again.
  * The layout is private to the library.  A packet whose segments do not fit
@@ -194,7 +197,7 @@ typedef struct {
                           the root, walk and shading in lockstep; packet = warps
                           of 32 consecutive rays, descents restarted at the
                           lowest common ancestor, walk and shading decoupled by
-                          a per-ray queue, tuned launch */
+                          a ring of segments per packet, tuned launch */
   int32_t compose_mode;/* neuvv_compose_mode */
 } neuvv_render_opts;
 
@@ -423,7 +426,7 @@ neuvv_status neuvv_gaussian_blur(const float *in, float *out, int32_t width, int
  * neuvv_render's packet kernel but reads only the w_sigma part of each leaf
  * record and evaluates no colour: out->alpha (required), depth, tau and nseg
  * (each optional) equal neuvv_render's for the same rays; out->rgb and
- * out->log are not used.  Launches one packet per warp without the tree's
+ * out->log are not used.  Launches one packet, or a part of one, per warp without the tree's
  * work counter, so it may run on another stream beside any call on the same
  * tree.  Built for K_pad 8 with degree 2 and K_pad 16 with degree 3 (else
  * NEUVV_ERR_UNSUPPORTED); other errors as neuvv_render. */
@@ -517,9 +520,9 @@ neuvv_status neuvv_log_read(const neuvv_out *saved, int64_t n, int32_t max_out, 
 neuvv_status neuvv_tree_set_packet_order(neuvv_tree *tree, int32_t order);
 
 /* Sets the packet kernels' launch explicitly instead of neuvv_autotune:
- * block (a multiple of 32 in [32, 256]), queue (a power of two in [1, 32]:
- * leaf segments a ray's walk may run ahead of its shading) and ready (1..32:
- * lanes with a queued segment that start a shading round).  Host only. */
+ * block (a multiple of 32 in [32, 256]), queue (a power of two in [1, 32];
+ * kept and reported, the ring of a packet has a fixed size) and ready (1..32:
+ * waiting segments that start a shading batch).  Host only. */
 neuvv_status neuvv_tree_set_launch(neuvv_tree *tree, int32_t block, int32_t queue, int32_t ready);
 
 /* Picks the packet kernels' launch -- block size, queue, ready count and the

