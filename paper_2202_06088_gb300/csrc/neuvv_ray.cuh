@@ -1,5 +1,6 @@
-// One ray through one VOctree: the forward integrator shared by the render and
-// compose kernels (Sec. 4.3 "Rendering"; Eq. volume-rendering).
+// Rays through one VOctree (Sec. 4.3 "Rendering"; Eq. volume-rendering): the
+// integrator of one thread per ray (the plain kernel), and the packets' ring and
+// batch shading shared by the packet forward, the adjoint and composition.
 #pragma once
 
 #include "neuvv_kernels.h"
@@ -14,21 +15,30 @@ struct RayResult {
   int nseg;      // composited segments
 };
 
-// Composites front to back along a started walk, stopping after the segment
-// that brings the transmittance below t_stop.  dn: unit direction in the
-// tree's frame (the view direction of the harmonics); u: frame coordinate;
-// t_base + dist_scale * t converts a walk distance t to the caller's frame.
+// One ray given in the tree's own frame, composited front to back up to and
+// including the segment that brings the transmittance below t_stop.  u: frame
+// coordinate.  One loop over walk steps with the sample inside it: lanes of a
+// warp keep stepping together and meet at the loop's head, where a search for
+// the next segment nested in a loop over segments made each lane wait for the
+// slowest search of every segment (1080p view of a depth-8 shell, 500,000 leaves,
+// K_pad 8 BF16: 0.86 of the time before the mirrored walk against 1.11 nested).
 template <int KP, int DEG, typename E>
-__device__ __forceinline__ void integrate_walk(const DevTree &tr, RayWalk &w,
-                                               const float dn[3], float u, float t_stop, int act, float t_base,
-                                               float dist_scale, RayResult &res) {
+__device__ __forceinline__ void integrate_ray(const DevTree &tr, const float o[3],
+                                              const float d[3], float u, float t_stop, int act, RayResult &res) {
+  res.C[0] = res.C[1] = res.C[2] = 0.f;
+  res.A = res.dnum = res.tau = 0.f;
+  res.nseg = 0;
+  RayWalk w;
+  float dn[3];
+  if (!walk_init(tr, o, d, w, dn)) return;
   RayConst<KP, DEG> rc;
   ray_const_basis<KP, DEG>(tr, u, rc);
   sh_real<DEG>(dn, rc.Y);
   float T = 1.f;
   uint32_t leaf;
   float t0, dt;
-  while (walk_next(tr, w, leaf, t0, dt)) {
+  while (w.alive) {
+    if (!walk_step(tr, w, leaf, t0, dt)) continue;
     LeafRecord<KP, DEG, E> rec;
     rec.load(tr, leaf);
     Sample<DEG> s;
@@ -41,31 +51,12 @@ __device__ __forceinline__ void integrate_walk(const DevTree &tr, RayWalk &w,
 #pragma unroll
       for (int ch = 0; ch < 3; ++ch) res.C[ch] = fmaf(wgt, s.c[ch], res.C[ch]);
       res.A += wgt;
-      res.dnum = fmaf(wgt, fmaf(dist_scale, fmaf(0.5f, dt, t0), t_base), res.dnum);
+      res.dnum = fmaf(wgt, w.t_base + fmaf(0.5f, dt, t0), res.dnum);
       res.tau += sd;
       T *= e;
       if (T < t_stop) break;
     }
   }
-}
-
-__device__ __forceinline__ void clear(RayResult &res) {
-  res.C[0] = res.C[1] = res.C[2] = 0.f;
-  res.A = 0.f;
-  res.dnum = 0.f;
-  res.tau = 0.f;
-  res.nseg = 0;
-}
-
-// One ray given in the tree's own frame (render kernels).
-template <int KP, int DEG, typename E>
-__device__ __forceinline__ void integrate_ray(const DevTree &tr, const float o[3],
-                                              const float d[3], float u, float t_stop, int act, RayResult &res) {
-  clear(res);
-  RayWalk w;
-  float dn[3];
-  if (!walk_init(tr, o, d, w, dn)) return;
-  integrate_walk<KP, DEG, E>(tr, w, dn, u, t_stop, act, w.t_base, 1.f, res);
 }
 
 // ---------------------------------------------------------------------------

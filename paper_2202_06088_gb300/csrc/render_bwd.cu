@@ -339,7 +339,7 @@ __device__ __forceinline__ bool adjoint_setup(const BwdArgs &a, long long i, Ray
   return true;
 }
 
-// One thread per ray, root descents (baseline).
+// One thread per ray (baseline); one loop over steps, as in integrate_ray.
 template <int KP, int DEG, typename E>
 __global__ void __launch_bounds__(256) render_bwd_plain_kernel(const __grid_constant__ BwdArgs a) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -353,7 +353,8 @@ __global__ void __launch_bounds__(256) render_bwd_plain_kernel(const __grid_cons
   sh_real<DEG>(dn, rc.Y);
   uint32_t leaf;
   float t0, dt;
-  while (st.count < st.target && walk_next(a.tr, w, leaf, t0, dt)) {
+  while (st.count < st.target && w.alive) {
+    if (!walk_step(a.tr, w, leaf, t0, dt)) continue;
     ++st.count;
     adjoint_sample<KP, DEG, E>(a, RegRows<KP>{rc.a, rc.b}, rc.Y, leaf, dt, st);
   }
