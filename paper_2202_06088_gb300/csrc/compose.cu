@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(256, packet_min_blocks<KP, DEG, E>())
   const long long stride = ((long long)gridDim.x * blockDim.x) >> 5;
   const int lane = threadIdx.x & 31;
   using Rec = LeafRecord<KP, DEG, E>;
-  using Shared = PacketShared<KP, Rec::kChunks>;
+  using Shared = PacketShared<KP, stage_chunks<KP, DEG, E>()>;
   const Shared sh(smem);
   const Shading shading{a.act, a.t_stop, nullptr, 0, nullptr, 0.f};
   long long p;
@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(256, packet_min_blocks<KP, DEG, E>())
 template <int KP, int DEG, typename E>
 static cudaError_t compose_one(const ComposeArgs &a, const LaunchCfg &cfg, cudaStream_t s) {
   if (a.rays.n == 0) return cudaSuccess;
-  const size_t sm = smem_bytes(cfg.block, KP, LeafRecord<KP, DEG, E>::kChunks, 0);
+  const size_t sm = smem_bytes(cfg.block, KP, stage_chunks<KP, DEG, E>(), 0);
   cudaError_t e;
   if (sm > 48 * 1024 && (e = cudaFuncSetAttribute(compose_kernel<KP, DEG, E>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                   (int)sm)) != cudaSuccess)

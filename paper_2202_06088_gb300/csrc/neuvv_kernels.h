@@ -276,26 +276,41 @@ constexpr int kPathWords = 16;
 __host__ __device__ inline int path_words(const DevTree &tr) { return tr.path_words; }
 constexpr int kPacketWords = 4 * kRing / 32 + 1 + 2 + 3;
 // Records of a batch staged in shared memory: 32 per warp, each of `chunks`
-// 16-byte chunks at an odd pitch, so that eight lanes reading one chunk of
-// their own records (a phase of a 16-byte load) hit distinct banks.  Smaller
-// records (K_pad 8, FP8) are read in place: staging them gains less than its
-// copies and the later shading cost (K_pad 8 BF16 composition 1044 against
-// 1100 us, a 128 x 128 FP32 view 78 against 83 us; K_pad 16 BF16 1080p view
-// 656 against 600 us).  So are records of more than 32 chunks (K_pad 32 in
-// FP32 with degree 3): eight warps' staging would not fit in an SM's shared
-// memory.
+// 16-byte chunks (0: none are) at an odd pitch, so that eight lanes reading one
+// chunk of their own records (a phase of a 16-byte load) hit distinct banks.
+// Staged are records of degree 3 and K_pad 8 or 16 of 16 chunks or more: their
+// colour part (90 entries) leaves a batch read in place no registers under 128.
+// The others' staging costs more, in copies, shared memory and so warps, than
+// its loads.  1080p view of a depth-8 shell of 500,000 leaves / of a depth-7 solid
+// of 160,000, time staged against in place:
+//   staged    K_pad 8 degree 3 FP32 (27 chunks) 0.76 / 0.96, K_pad 16 degree 3 FP32
+//             (31) 0.80 / 0.98 and BF16 (16) 0.96 / 1.07 (0.92 on a depth-9 shell)
+//   in place  K_pad 16 degree 2 FP32 (19) 1.16 / 1.30, K_pad 32 degree 1 FP32 (20) 1.14 / 1.35,
+//             degree 2 FP32 (27) 1.34 / 1.53, degree 3 BF16 (20) 1.10 / 1.39,
+//             K_pad 8 degree 3 BF16 (14) 1.00 / 1.09
 constexpr int kMinStage = 16, kMaxStage = 32;
-__host__ __device__ constexpr bool staged(int chunks) { return chunks >= kMinStage && chunks <= kMaxStage; }
-__host__ __device__ constexpr int stage_pitch(int chunks) { return staged(chunks) ? (chunks | 1) : 0; }
+template <int KP, int DEG, typename E>
+__host__ __device__ constexpr int stage_chunks() {
+  constexpr int c = LeafRecord<KP, DEG, E>::kChunks;
+  return DEG == 3 && KP <= 16 && c >= kMinStage && c <= kMaxStage ? c : 0;
+}
+__host__ __device__ constexpr int stage_pitch(int chunks) { return chunks ? (chunks | 1) : 0; }
 inline size_t smem_bytes(int block, int KP, int chunks, int path) {
   return (size_t)block * (kPacketWords + 4 * stage_pitch(chunks) + 2 * KP + path) * sizeof(float);
 }
+// Staging also has to leave more than 8 warps to an SM (228 KB, 1 KB of it per
+// block taken by the system): large blocks whose records no longer fit twice
+// read them in place (blocks of 256, K_pad 16 degree 3 BF16, the views above: 1.21
+// and 1.34 staged against in place; blocks of 128, 12 warps: 0.94 and 1.14).
+inline bool stage_fits(int block, size_t smem) { return (233472 / (smem + 1024)) * (block / 32) > 8; }
 constexpr int kMaxQueue = 32;
 // Packet kernels are latency bound: two 256-thread blocks per SM (128
-// registers a thread) keep enough warps resident; records of more than
-// kMaxStage chunks need the registers of one block per SM instead.
+// registers a thread) keep enough warps resident; records of more than 32
+// chunks (K_pad 32 FP32 with degree 3) need the registers of one block per SM
+// instead.  K_pad 32 FP32 with degree 2 (27 chunks), the views above: 0.69 and 0.77
+// of the time with 255 registers.
 template <int KP, int DEG, typename E>
-constexpr int packet_min_blocks() { return LeafRecord<KP, DEG, E>::kChunks <= kMaxStage ? 2 : 1; }
+constexpr int packet_min_blocks() { return LeafRecord<KP, DEG, E>::kChunks <= 32 ? 2 : 1; }
 constexpr int kMaxDepth = 14;
 
 }  // namespace neuvv

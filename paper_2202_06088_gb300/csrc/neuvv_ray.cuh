@@ -81,10 +81,10 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Pointers into a packet kernel's dynamic shared memory (kPacketWords); CHUNKS:
-// 16-byte chunks of the records that are staged.
+// 16-byte chunks of the records that are staged (0: none are).
 template <int KP, int CHUNKS>
 struct PacketShared {
-  static constexpr bool kStaged = staged(CHUNKS);
+  static constexpr bool kStaged = CHUNKS > 0;
   static constexpr int kPitch = stage_pitch(CHUNKS);
   uint4 *ring;      // [kRing] leaf, chord, distance of its middle, lane of the ray
   uint4 *stage;     // [32][kPitch] records of a batch
@@ -112,7 +112,6 @@ struct PacketShared {
   // own record 16 bytes at a time touches 32 lines per load; those wavefronts
   // kept L1 at 56 % of its peak in the 1080p forward, against 19 % now).  The
   // copies run while the rays walk on.  Lanes without an entry pass leaf 0.
-  // (0 chunks: nothing is ever staged)
   static constexpr int kGroup = CHUNKS > 16 ? 32 : (CHUNKS > 8 ? 16 : 8);
   __device__ __forceinline__ void stage_records(const void *base, uint32_t rec_bytes, uint32_t leaf, int count) const {
     const int lane = threadIdx.x & 31, c = lane % kGroup, r0 = lane / kGroup;
@@ -171,7 +170,7 @@ __host__ __device__ constexpr bool density_only(int shade) { return shade == kSh
 template <int KP, int DEG, typename E, int kShade>
 __host__ __device__ constexpr int shade_chunks() {
   // slice rows are small, and a density-only batch reads few chunks: in place
-  return kShade == kShadeSlice || density_only(kShade) ? 0 : LeafRecord<KP, DEG, E>::kChunks;
+  return kShade == kShadeSlice || density_only(kShade) ? 0 : stage_chunks<KP, DEG, E>();
 }
 struct Shading {
   int act;

@@ -65,14 +65,14 @@ __device__ __forceinline__ void write_miss(const DevOut &out, long long i) {
 // one long ray among finished ones shades up to 32 of its own segments at once.
 // Descents restart at the lowest common ancestor of successive cells (path per
 // thread in shared memory); basis rows and directions live in shared memory.
-template <int KP, int DEG, typename E, int kShade = kShadeTree>
+// CHUNKS: chunks of the records that are staged (0: read in place).
+template <int KP, int DEG, typename E, int kShade, int CHUNKS>
 __device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, int split, int part, long long n_live,
                                                int ready) {
   extern __shared__ __align__(16) uint32_t smem[];
   const DevTree &tr = a.tr;
   const int lane = threadIdx.x & 31;
-  constexpr int kChunks = shade_chunks<KP, DEG, E, kShade>();
-  using Shared = PacketShared<KP, kChunks>;
+  using Shared = PacketShared<KP, CHUNKS>;
   const Shared sh(smem);
   const PathRef pr{sh.path, sh.stride};
   // the warp holds 32 >> split of the packet's rays, in its first lanes
@@ -211,7 +211,7 @@ __device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, i
 // Packet forward kernel.  With a work counter the grid is persistent: each
 // warp takes the next 32-ray packet from the counter when it finishes one, so
 // a long ray holds up only its own warp, not the other warps of its block.
-template <int KP, int DEG, typename E, int kShade = kShadeTree>
+template <int KP, int DEG, typename E, int kShade, int CHUNKS>
 __global__ void __launch_bounds__(256, density_only(kShade) ? 4 : packet_min_blocks<KP, DEG, E>())
     render_packet_kernel(const __grid_constant__ FwdArgs a, int ready) {
   // one packet per warp of the grid, or (with a work counter) packets pulled
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(256, density_only(kShade) ? 4 : packet_min_blo
       split = (int)(v >> 20) & 3;
       part = (int)(v >> 24);
     }
-    packet_forward<KP, DEG, E, kShade>(a, pk, split, part, n_live, ready);
+    packet_forward<KP, DEG, E, kShade, CHUNKS>(a, pk, split, part, n_live, ready);
     __syncwarp();
     if (!a.work) break;
     unsigned long long q = 0;
@@ -408,20 +408,21 @@ constexpr int kTriageLevel = 5;
 // that the call allows: of rays with a log in which the packets are taken as
 // given (n < 2^32), of packets without a log on trees of depth 8 to 10 (with a
 // brick map) whose bricks are less than half full.
-template <int KP, int DEG, typename E, int kShade>
+template <int KP, int DEG, typename E, int kShade, int CHUNKS = shade_chunks<KP, DEG, E, kShade>()>
 static cudaError_t packet_launch(FwdArgs a, const LaunchCfg &cfg, cudaStream_t s) {
   if (a.rays.n == 0) return cudaSuccess;
   const long long n_packets = (a.rays.n + 31) >> 5;
   const int warps = cfg.block / 32;
-  const size_t sm = smem_bytes(cfg.block, KP, shade_chunks<KP, DEG, E, kShade>(), path_words(a.tr));
+  const size_t sm = smem_bytes(cfg.block, KP, CHUNKS, path_words(a.tr));
+  if constexpr (CHUNKS > 0)
+    if (!stage_fits(cfg.block, sm)) return packet_launch<KP, DEG, E, kShade, 0>(a, cfg, s);
+  const auto kernel = render_packet_kernel<KP, DEG, E, kShade, CHUNKS>;
   cudaError_t e;
-  if (sm > 48 * 1024 && (e = cudaFuncSetAttribute(render_packet_kernel<KP, DEG, E, kShade>,
-                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
+  if (sm > 48 * 1024 &&
+      (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
     return e;
   int per_sm = 0;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, render_packet_kernel<KP, DEG, E, kShade>, cfg.block,
-                                                         sm)) != cudaSuccess)
-    return e;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, cfg.block, sm)) != cudaSuccess) return e;
   const long long want = (long long)(per_sm > 0 ? per_sm : 1) * cfg.num_sms;  // resident blocks
   const long long resident = want * warps;
   if (!a.log.n_chunks)
@@ -454,7 +455,7 @@ static cudaError_t packet_launch(FwdArgs a, const LaunchCfg &cfg, cudaStream_t s
   if (a.n_live && (e = cudaMemsetAsync(a.log.heads, 0xFF, (size_t)((char *)(a.log.key + n_packets) - (char *)a.log.heads),
                                        s)) != cudaSuccess)
     return e;
-  render_packet_kernel<KP, DEG, E, kShade><<<(unsigned)grid, cfg.block, sm, s>>>(a, cfg.ready);
+  kernel<<<(unsigned)grid, cfg.block, sm, s>>>(a, cfg.ready);
   return cudaGetLastError();
 }
 
