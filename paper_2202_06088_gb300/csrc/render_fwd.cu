@@ -211,8 +211,16 @@ __device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, i
 // Packet forward kernel.  With a work counter the grid is persistent: each
 // warp takes the next 32-ray packet from the counter when it finishes one, so
 // a long ray holds up only its own warp, not the other warps of its block.
+// Registers: those that packet_min_blocks leaves a block of 256 threads, and 96
+// for a density-only shading.  Held to 64 that one spilled the walk's state;
+// with 80 the larger K_pad were slower, with 128 the smaller.  Two 1280 x 720
+// views of density alone, with 64 -> 96, against the kernel before batches
+// (128): depth-8 shell of 500,000 leaves K_pad 16 FP32 degree 3 1.05 -> 0.80, K_pad 8
+// BF16 0.91 -> 0.87; depth-7 solid of 160,000 1.32 -> 0.99 and 1.06 -> 1.02.
+template <int KP, int DEG, typename E, int kShade>
+constexpr int packet_registers() { return density_only(kShade) ? 96 : (packet_min_blocks<KP, DEG, E>() == 2 ? 128 : 255); }
 template <int KP, int DEG, typename E, int kShade, int CHUNKS>
-__global__ void __launch_bounds__(256, density_only(kShade) ? 4 : packet_min_blocks<KP, DEG, E>())
+__global__ void __maxnreg__((packet_registers<KP, DEG, E, kShade>()))
     render_packet_kernel(const __grid_constant__ FwdArgs a, int ready) {
   // one packet per warp of the grid, or (with a work counter) packets pulled
   // one after another until the counter passes the last
