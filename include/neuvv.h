@@ -134,8 +134,8 @@ typedef struct {
   int32_t packet_block;     /* packet kernels: threads per block */
   int32_t packet_queue;     /* packet kernels: as set by the caller (a packet's segments wait in
                                one ring, whose size is fixed) */
-  int32_t packet_ready;     /* packet kernels: waiting segments of a packet that start a shading
-                               batch (all three set by neuvv_autotune) */
+  int32_t packet_ready;     /* packet kernels: as set by the caller (a shading batch starts at 32
+                               waiting segments; all three set by neuvv_autotune) */
   int32_t packet_order;     /* packet forward with a segment log: NEUVV_ORDER_* (neuvv_autotune) */
   int32_t packet_tiles;     /* pixel tile of a 32-ray packet of camera rays, NEUVV_TILES_*
                                (neuvv_autotune_tiles; default 8x4) */
@@ -520,12 +520,13 @@ neuvv_status neuvv_log_read(const neuvv_out *saved, int64_t n, int32_t max_out, 
 neuvv_status neuvv_tree_set_packet_order(neuvv_tree *tree, int32_t order);
 
 /* Sets the packet kernels' launch explicitly instead of neuvv_autotune:
- * block (a multiple of 32 in [32, 256]), queue (a power of two in [1, 32];
- * kept and reported, the ring of a packet has a fixed size) and ready (1..32:
- * waiting segments that start a shading batch).  Host only. */
+ * block (a multiple of 32 in [32, 256]), queue (a power of two in [1, 32])
+ * and ready (1..32).  queue and ready are checked, kept and reported: a packet's
+ * segments wait in one ring of fixed size, and its batches start at 32 of them.
+ * Host only. */
 neuvv_status neuvv_tree_set_launch(neuvv_tree *tree, int32_t block, int32_t queue, int32_t ready);
 
-/* Picks the packet kernels' launch -- block size, queue, ready count and the
+/* Picks the packet kernels' launch -- block size and the
  * forward's packet order (NEUVV_ORDER_*) -- by timing candidates with the
  * packet forward (with a segment log of 64 bytes per ray) on a sample of
  * rays (the first min(n, 2^20)); the fastest is stored in the tree.  The

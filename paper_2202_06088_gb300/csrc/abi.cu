@@ -1558,7 +1558,7 @@ neuvv_status neuvv_autotune(neuvv_tree *t, const neuvv_rays *sample, float time,
   float best_t = 1e30f;
   std::vector<neuvv_tune_entry> table;
   struct Cand { int block, queue, ready; };
-  const Cand cands[] = {{64, 8, 32}, {64, 8, 24}, {64, 8, 16}, {128, 8, 32}, {32, 8, 32}};
+  const Cand cands[] = {{64, 8, 32}, {128, 8, 32}, {32, 8, 32}, {256, 8, 32}};
   for (int order = NEUVV_ORDER_AS_GIVEN; order <= NEUVV_ORDER_BY_RAY && s == NEUVV_OK; ++order)
     for (const Cand &c : cands) {
       t->packet = saved;

@@ -251,10 +251,10 @@ __global__ void __launch_bounds__(256, packet_min_blocks<KP, DEG, E>())
           if (!Shared::kStaged) Rec::prefetch_l2(tr, leaf);
         }
         count += __popc(finds);
-        if (count < 32 && __any_sync(kFull, walking)) continue;
+        if (count < kBatch && __any_sync(kFull, walking)) continue;
         // batches as in the packet forward: shaded one batch late when staged
         __syncwarp();
-        const int batch = min(count, 32);
+        const int batch = min(count, kBatch);
         const bool next_has = lane < batch;
         const uint4 next_en = sh.ring[(head + lane) & (kRing - 1)];
         if (!Shared::kStaged) {

@@ -487,7 +487,7 @@ cudaError_t launch_packet_order(const DevTree &tr, const DevRays &rays, const Sa
 // the forward's segment count.  Not inlined: its state does not add to the
 // registers of the replay, which most packets take.
 template <int KP, int DEG, typename E>
-__device__ __noinline__ void adjoint_walk_packet(const BwdArgs &a, long long i, bool live, int ready) {
+__device__ __noinline__ void adjoint_walk_packet(const BwdArgs &a, long long i, bool live) {
   extern __shared__ __align__(16) uint32_t smem[];
   const DevTree &tr = a.tr;
   const int lane = threadIdx.x & 31;
@@ -520,10 +520,10 @@ __device__ __noinline__ void adjoint_walk_packet(const BwdArgs &a, long long i, 
       sh.ring[slot] = make_uint4(leaf, __float_as_uint(dt), 0u, lane);
     }
     count += __popc(finds);
-    if (count < ready && __any_sync(kFull, walking)) continue;
+    if (count < kBatch && __any_sync(kFull, walking)) continue;
     if (count == 0) break;
     __syncwarp();
-    const int batch = min(count, 32);
+    const int batch = min(count, kBatch);
     const uint4 en = sh.ring[(head + lane) & (kRing - 1)];
     head += batch;
     count -= batch;
@@ -567,7 +567,7 @@ struct LogCursor {
 // to 20 chunks, read in place, fit in 128 registers; larger ones take 255.
 template <int KP, int DEG, typename E>
 __global__ void __launch_bounds__(256, LeafRecord<KP, DEG, E>::kChunks <= 20 ? 2 : 1)
-    render_bwd_packet_kernel(const __grid_constant__ BwdArgs a, int ready) {
+    render_bwd_packet_kernel(const __grid_constant__ BwdArgs a) {
   extern __shared__ __align__(16) uint32_t smem[];
   const DevTree &tr = a.tr;
   const int lane = threadIdx.x & 31;
@@ -588,7 +588,7 @@ __global__ void __launch_bounds__(256, LeafRecord<KP, DEG, E>::kChunks <= 20 ? 2
                           : pos;
   const uint32_t head = logged ? __ldg(a.log.heads + pk) : kNoLog;  // warp-uniform
   if (head == kNoLog) {
-    adjoint_walk_packet<KP, DEG, E>(a, i, live, ready);
+    adjoint_walk_packet<KP, DEG, E>(a, i, live);
     return;
   }
   RayWalk w;
@@ -962,7 +962,7 @@ static cudaError_t bwd_one(bool packet, const BwdArgs &a, const LaunchCfg &cfg, 
       e = cudaMemcpyAsync(a.gws.cur, a.gws.off, (size_t)(nl + 1) * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s);
       if (e != cudaSuccess) return e;
     }
-    render_bwd_packet_kernel<KP, DEG, E><<<(unsigned)blocks, cfg.block, sm, s>>>(b, cfg.ready);
+    render_bwd_packet_kernel<KP, DEG, E><<<(unsigned)blocks, cfg.block, sm, s>>>(b);
     if (gather) {
       // the per-leaf sums over each leaf's run
       AdamArgs ad{};

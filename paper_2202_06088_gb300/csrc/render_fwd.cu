@@ -57,7 +57,7 @@ __device__ __forceinline__ void write_miss(const DevOut &out, long long i) {
 // consecutive rays (an 8x4 pixel tile when the caller orders rays that way).
 // Walking and shading are decoupled: in every iteration of one warp-uniform
 // loop each lane takes at most one walk step, and the occupied-leaf segments
-// found join the packet's ring.  Once `ready` segments wait, or no ray can step
+// found join the packet's ring.  Once kBatch segments wait, or no ray can step
 // any further, the warp shades a batch of up to 32 of them, one per lane
 // whichever rays they belong to, and each ray composites its own entries in
 // order (a shuffle of the seven values that compositing needs per entry).
@@ -67,8 +67,7 @@ __device__ __forceinline__ void write_miss(const DevOut &out, long long i) {
 // thread in shared memory); basis rows and directions live in shared memory.
 // CHUNKS: chunks of the records that are staged (0: read in place).
 template <int KP, int DEG, typename E, int kShade, int CHUNKS>
-__device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, int split, int part, long long n_live,
-                                               int ready) {
+__device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, int split, int part, long long n_live) {
   extern __shared__ __align__(16) uint32_t smem[];
   const DevTree &tr = a.tr;
   const int lane = threadIdx.x & 31;
@@ -127,11 +126,11 @@ __device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, i
       }
     }
     count += __popc(finds);
-    if (count < ready && __any_sync(kFull, walking)) continue;
+    if (count < kBatch && __any_sync(kFull, walking)) continue;
     // the next batch: with staging its records are on their way while the
     // rays walk on, and it is shaded when the one after it is complete
     __syncwarp();
-    const int batch = min(count, 32);
+    const int batch = min(count, kBatch);
     const bool next_has = lane < batch;
     const uint4 next_en = sh.ring[(head + lane) & (kRing - 1)];
     if (!Shared::kStaged) {
@@ -221,7 +220,7 @@ template <int KP, int DEG, typename E, int kShade>
 constexpr int packet_registers() { return density_only(kShade) ? 96 : (packet_min_blocks<KP, DEG, E>() == 2 ? 128 : 255); }
 template <int KP, int DEG, typename E, int kShade, int CHUNKS>
 __global__ void __maxnreg__((packet_registers<KP, DEG, E, kShade>()))
-    render_packet_kernel(const __grid_constant__ FwdArgs a, int ready) {
+    render_packet_kernel(const __grid_constant__ FwdArgs a) {
   // one packet per warp of the grid, or (with a work counter) packets pulled
   // one after another until the counter passes the last
   const int lane = threadIdx.x & 31;
@@ -258,7 +257,7 @@ __global__ void __maxnreg__((packet_registers<KP, DEG, E, kShade>()))
       split = (int)(v >> 20) & 3;
       part = (int)(v >> 24);
     }
-    packet_forward<KP, DEG, E, kShade, CHUNKS>(a, pk, split, part, n_live, ready);
+    packet_forward<KP, DEG, E, kShade, CHUNKS>(a, pk, split, part, n_live);
     __syncwarp();
     if (!a.work) break;
     unsigned long long q = 0;
@@ -463,7 +462,7 @@ static cudaError_t packet_launch(FwdArgs a, const LaunchCfg &cfg, cudaStream_t s
   if (a.n_live && (e = cudaMemsetAsync(a.log.heads, 0xFF, (size_t)((char *)(a.log.key + n_packets) - (char *)a.log.heads),
                                        s)) != cudaSuccess)
     return e;
-  kernel<<<(unsigned)grid, cfg.block, sm, s>>>(a, cfg.ready);
+  kernel<<<(unsigned)grid, cfg.block, sm, s>>>(a);
   return cudaGetLastError();
 }
 
