@@ -159,12 +159,12 @@ DevRays dev_rays(const neuvv_rays *r, float t) {
 
 // Device view of a caller's segment log buffer (layout private to the
 // library): 64-byte header, heads, key and order [n_packets], perm [n_rays],
-// the sort bins, next [n_chunks], then leaf, chord and lane planes of n_chunks x
-// kLogRounds x 32 entries.  n_chunks = 0 when the buffer is absent or too
-// small for one chunk.  *chunk_bytes (nullable) receives the bytes from the
+// the sort bins, next [n_chunks], then leaf, chord and (wide) lane planes of
+// n_chunks x kLogRounds x 32 entries.  n_chunks = 0 when the buffer is absent or
+// too small for one chunk.  *chunk_bytes (nullable) receives the bytes from the
 // start of next[] to the end of the buffer (scratch for a ray order before
 // the forward fills the chunks).
-SampleLog log_view(void *base, int64_t bytes, int64_t n_rays, int64_t *chunk_bytes = nullptr) {
+SampleLog log_view(void *base, int64_t bytes, int64_t n_rays, bool wide, int64_t *chunk_bytes = nullptr) {
   SampleLog l;
   std::memset(&l, 0, sizeof l);
   if (chunk_bytes) *chunk_bytes = 0;
@@ -176,7 +176,7 @@ SampleLog log_view(void *base, int64_t bytes, int64_t n_rays, int64_t *chunk_byt
   const int64_t pk_bytes = (4 * n_packets + 15) / 16 * 16;
   const int64_t perm_bytes = (4 * n_rays + 15) / 16 * 16;
   const int64_t fixed = 64 + 3 * pk_bytes + perm_bytes + 4 * kSortBins;
-  const int64_t per_chunk = 4 + (int64_t)kLogRounds * 32 * 9;
+  const int64_t per_chunk = 4 + (int64_t)kLogRounds * 32 * (wide ? 9 : 8);
   const int64_t avail = bytes - fixed - 16;
   if (avail < per_chunk) return l;
   int64_t nc = avail / per_chunk;
@@ -190,11 +190,13 @@ SampleLog log_view(void *base, int64_t bytes, int64_t n_rays, int64_t *chunk_byt
   const int64_t leaf_off = (fixed + 4 * nc + 15) / 16 * 16;
   l.leaf = reinterpret_cast<uint32_t *>(p + leaf_off);
   l.dt = reinterpret_cast<float *>(p + leaf_off + nc * kLogRounds * 32 * 4);
-  l.lane = reinterpret_cast<uint8_t *>(l.dt + nc * kLogRounds * 32);
+  if (wide) l.lane = reinterpret_cast<uint8_t *>(l.dt + nc * kLogRounds * 32);
   l.n_chunks = (uint32_t)nc;
   if (chunk_bytes) *chunk_bytes = bytes - fixed;
   return l;
 }
+
+bool wide_log(const neuvv_tree *t) { return t->info.n_leaves > kPackedLeaves; }
 
 neuvv_status check_log(const neuvv_out *out) {
   if (out && out->log && (((uintptr_t)out->log & 15) != 0 || out->log_bytes < 0))
@@ -810,7 +812,7 @@ neuvv_status neuvv_render(const neuvv_tree *t, const neuvv_rays *rays, float tim
   a.work = packet && cfg.dynamic_queue ? t->work + 0 : nullptr;
   a.queue = t->queue;
   int64_t chunk_bytes = 0;
-  a.log = packet ? log_view(out->log, out->log_bytes, rays->n, &chunk_bytes) : log_view(nullptr, 0, 0);
+  a.log = packet ? log_view(out->log, out->log_bytes, rays->n, wide_log(t), &chunk_bytes) : SampleLog{};
   a.slice = nullptr;
   a.slice_stride = 0;
   a.edits = nullptr;
@@ -858,7 +860,7 @@ neuvv_status neuvv_render_alpha(const neuvv_tree *t, const neuvv_rays *rays, flo
   a.t_stop = opts->t_stop;
   a.act = opts->color_act;
   a.work = nullptr;
-  a.log = log_view(nullptr, 0, 0);
+  a.log = SampleLog{};
   a.slice = nullptr;
   a.slice_stride = 0;
   a.edits = nullptr;
@@ -914,7 +916,7 @@ neuvv_status neuvv_render_slice(const neuvv_tree *t, const float *slice, int32_t
   const LaunchCfg &cfg = t->packet;
   a.work = cfg.dynamic_queue ? t->work + 0 : nullptr;
   a.queue = t->queue;
-  a.log = log_view(nullptr, 0, 0);
+  a.log = SampleLog{};
   a.slice = slice;
   a.slice_stride = slice_stride;
   a.edits = nullptr;
@@ -955,7 +957,7 @@ neuvv_status prepare_backward(const neuvv_tree *t, const neuvv_rays *rays, float
   a.touched = touched;
   a.t_stop = opts->t_stop;
   a.act = opts->color_act;
-  a.log = log_view(saved->log, saved->log_bytes, rays->n);
+  a.log = log_view(saved->log, saved->log_bytes, rays->n, wide_log(t));
   const bool packet = opts->kernel != NEUVV_KERNEL_PLAIN;
   a.key_order = 1;
   a.gws = packet && a.log.n_chunks ? t->gws : GatherWs{};
@@ -1293,7 +1295,7 @@ neuvv_status neuvv_render_edit(const neuvv_tree *t, const neuvv_rays *rays, floa
   const LaunchCfg &cfg = t->packet;
   a.work = cfg.dynamic_queue ? t->work + 0 : nullptr;
   a.queue = t->queue;
-  a.log = log_view(nullptr, 0, 0);
+  a.log = SampleLog{};
   a.edits = edits;
   a.edit_beta = beta;
   cudaError_t e = clear_log(out, st);
@@ -1445,8 +1447,10 @@ neuvv_status neuvv_log_read(const neuvv_out *saved, int64_t n, int32_t max_out, 
   if (n > 0 && (!count || (max_out > 0 && (!leaf || !chord))))
     return fail(NEUVV_ERR_INVALID_ARG, "output pointer is NULL");
   if (n == 0) return NEUVV_OK;
-  const SampleLog l = log_view(saved->log, saved->log_bytes, n);
-  cudaError_t e = launch_log_read(l, (long long)n, saved->nseg, max_out, leaf, chord, count, (cudaStream_t)stream);
+  const SampleLog packed = log_view(saved->log, saved->log_bytes, n, false);
+  const SampleLog wide = log_view(saved->log, saved->log_bytes, n, true);
+  cudaError_t e = launch_log_read(packed, wide, (long long)n, saved->nseg, max_out, leaf, chord, count,
+                                  (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "log read launch");
   return NEUVV_OK;
 }

@@ -24,9 +24,10 @@ struct LaunchCfg {
 
 // Segment log of the packet forward (device view of neuvv_out.log).  Chunks
 // of kLogRounds shading rounds x 32 slots hold (leaf, chord, lane of the
-// ray) per composited segment, a ray's segments in order, leaf = kEmpty in a
-// slot without one; a packet's chunks are linked
-// from heads[packet] through next[].  heads[packet] = kNoLog: not logged
+// ray) per composited segment, a ray's segments in order, kEmpty in the leaf
+// plane of a slot without one.  Trees of up to kPackedLeaves leaves keep leaf and
+// lane in one word (8 bytes a slot); larger ones have a lane plane (9 bytes).
+// A packet's chunks are linked from heads[packet] through next[].  heads[packet] = kNoLog: not logged
 // (replay by walking).  Header: chunk counter (u64), then n_chunks, rounds,
 // n_rays (i64), a valid word and a permuted word, all written by the forward
 // that fills it.  Packets are formed from positions: position p holds ray
@@ -36,18 +37,22 @@ constexpr uint32_t kNoLog = 0xFFFFFFFFu;
 struct SampleLog {
   unsigned long long *counter;
   uint32_t *header;   // [0] n_chunks, [1] rounds, [2..3] n_rays, [4] valid, [5] permuted, [6..7] n_live:
-                      // positions from n_live on hold rays that miss the tree's box ([8] counts them)
+                      // positions from n_live on hold rays that miss the tree's box ([8] counts them),
+                      // [9] layout()
   uint32_t *perm;     // [n_rays] ray of each position (when permuted)
   uint32_t *heads;    // [n_packets]
   uint32_t *key;      // [n_packets] first leaf the packet shaded (kNoKey: none)
   uint32_t *order;    // [n_packets] packets sorted by key (filled by the adjoint)
   uint32_t *bins;     // [kSortBins] counting-sort scratch
   uint32_t *next;     // [n_chunks]
-  uint32_t *leaf;     // [n_chunks][kLogRounds][32]
+  uint32_t *leaf;     // [n_chunks][kLogRounds][32] leaf << 5 | lane, or the leaf where there is a lane plane
   float *dt;          // [n_chunks][kLogRounds][32]
-  uint8_t *lane;      // [n_chunks][kLogRounds][32] the packet's lane whose ray a slot belongs to
+  uint8_t *lane;      // [n_chunks][kLogRounds][32] the packet's lane whose ray a slot belongs to (null: packed)
   uint32_t n_chunks;  // 0: no log
+  __host__ __device__ uint32_t layout() const { return lane ? 2u : 1u; }
 };
+// A packed word names a leaf below 2^27 - 1, so that none reads kEmpty.
+constexpr long long kPackedLeaves = (1 << 27) - 1;
 constexpr uint32_t kNoKey = 0xFFFFFFFFu;
 // Bins of the counting sort that orders the adjoint's packets by key (leaf
 // ids follow the Morton order of the leaves, so a bin is a compact region).
@@ -252,9 +257,10 @@ cudaError_t launch_render_slice(int DEG, const FwdArgs &a, const LaunchCfg &cfg,
 // Device address of the static work counter used by neuvv_compose_noalloc in
 // the current CUDA context (looked up on first use per context).
 cudaError_t noalloc_queue(unsigned long long **out);
-// Decodes a packet forward's segment log into per-ray (leaf, chord) lists.
-cudaError_t launch_log_read(const SampleLog &l, long long n_rays, const int *nseg, int max_out, int *leaf,
-                            float *chord, int *count, cudaStream_t s);
+// Decodes a packet forward's segment log into per-ray (leaf, chord) lists
+// (both views of the caller's buffer).
+cudaError_t launch_log_read(const SampleLog &packed, const SampleLog &wide, long long n_rays, const int *nseg,
+                            int max_out, int *leaf, float *chord, int *count, cudaStream_t s);
 cudaError_t launch_adam(float *master, float *m, float *v, void *storage, DType dt, int storage_stride, float *grad,
                         const unsigned int *touched, long long n_leaves, int stride_f32, int rec_len, int kp,
                         float lr, float b1, float b2, float eps, float c1, float c2, cudaStream_t s);

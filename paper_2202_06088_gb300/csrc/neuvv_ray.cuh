@@ -72,6 +72,24 @@ __device__ __forceinline__ void integrate_ray(const DevTree &tr, const float o[3
 // ---------------------------------------------------------------------------
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
+// Whether a segment log was written by a forward over n rays.
+__device__ __forceinline__ bool log_matches(const SampleLog &l, long long n) {
+  return __ldg(l.header + 4) == 1u && __ldg(l.header) == l.n_chunks && __ldg(l.header + 1) == (uint32_t)kLogRounds &&
+         __ldg(l.header + 2) == (uint32_t)(n & 0xFFFFFFFFll) && __ldg(l.header + 3) == (uint32_t)(n >> 32) &&
+         __ldg(l.header + 9) == l.layout();
+}
+// Leaf and lane of a slot of the log.
+struct LogWord {
+  uint32_t leaf;
+  int lane;
+  bool empty;
+};
+__device__ __forceinline__ LogWord log_word(const SampleLog &l, size_t slot) {
+  const uint32_t w = __ldcs(l.leaf + slot);
+  if (l.lane) return LogWord{w, (int)__ldcs(l.lane + slot) & 31, w == kEmpty};
+  return LogWord{w >> 5, (int)(w & 31u), w == kEmpty};
+}
+
 // Asynchronous 16-byte copy from global to shared memory (past L1), and the
 // wait for this thread's copies.
 __device__ __forceinline__ void cp_async16(void *dst, const void *src) {

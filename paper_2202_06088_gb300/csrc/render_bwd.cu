@@ -312,12 +312,6 @@ __device__ __forceinline__ void adjoint_batch(const BwdArgs &a, const Sh &sh, ui
   __syncwarp();  // the shared results are rewritten by the next batch
 }
 
-// Whether a segment log was written by a forward over these rays.
-__device__ __forceinline__ bool log_matches(const SampleLog &l, long long n) {
-  return __ldg(l.header + 4) == 1u && __ldg(l.header) == l.n_chunks && __ldg(l.header + 1) == (uint32_t)kLogRounds &&
-         __ldg(l.header + 2) == (uint32_t)(n & 0xFFFFFFFFll) && __ldg(l.header + 3) == (uint32_t)(n >> 32);
-}
-
 // Sets up the replay of ray i; false when the ray has nothing to replay.
 __device__ __forceinline__ bool adjoint_setup(const BwdArgs &a, long long i, RayWalk &w, float dn[3], float &t,
                                               AdjState &st) {
@@ -549,10 +543,11 @@ struct LogCursor {
     LogEntry e{kEmpty, chunk, 0.f, 0, false};
     if (chunk >= l.n_chunks) return e;
     const size_t slot = ((size_t)chunk * kLogRounds + round) * 32 + (threadIdx.x & 31);
-    e.leaf = __ldcs(l.leaf + slot);
+    const LogWord w = log_word(l, slot);
+    e.leaf = w.leaf;
     e.dt = __ldcs(l.dt + slot);
-    e.owner = (int)__ldcs(l.lane + slot) & 31;
-    e.has = e.leaf != kEmpty && ((rays >> e.owner) & 1u);
+    e.owner = w.lane;
+    e.has = !w.empty && ((rays >> e.owner) & 1u);
     if (++round == kLogRounds) {
       round = 0;
       chunk = __ldg(l.next + chunk);
@@ -644,8 +639,9 @@ __global__ void __launch_bounds__(256) leaf_count_kernel(const __grid_constant__
   const int lane = threadIdx.x & 31;
   const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
   for (long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w * 32 < n_slots; w += warps) {
-    const uint32_t leaf = __ldcs(a.log.leaf + w * 32 + lane);
-    const bool has = leaf < n_leaves;
+    const uint32_t word = __ldcs(a.log.leaf + w * 32 + lane);
+    const uint32_t leaf = a.log.lane ? word : word >> 5;
+    const bool has = word != kEmpty && leaf < n_leaves;
     const unsigned grp = __match_any_sync(0xFFFFFFFFu, has ? leaf : kEmpty);
     if (has && lane == __ffs(grp) - 1) atomicAdd(a.gws.off + leaf, (uint32_t)__popc(grp));
   }

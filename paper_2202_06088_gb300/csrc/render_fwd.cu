@@ -170,9 +170,9 @@ __device__ __forceinline__ void packet_forward(const FwdArgs &a, long long pk, i
         // the entries that were composited (a ray that ended drops its later ones)
         const bool keep = (__reduce_or_sync(kFull, kept) >> lane) & 1u;
         const size_t slot = ((size_t)chunk * kLogRounds + round) * 32 + lane;
-        __stcs(a.log.leaf + slot, keep ? en.x : kEmpty);
+        __stcs(a.log.leaf + slot, !keep ? kEmpty : (a.log.lane ? en.x : (en.x << 5 | (en.w & 31u))));
         __stcs(a.log.dt + slot, keep ? __uint_as_float(en.y) : 0.f);
-        a.log.lane[slot] = (uint8_t)en.w;
+        if (a.log.lane) a.log.lane[slot] = (uint8_t)en.w;
         ++round;
       }
     }
@@ -235,6 +235,7 @@ __global__ void __maxnreg__((packet_registers<KP, DEG, E, kShade>()))
     a.log.header[3] = (uint32_t)(a.rays.n >> 32);
     a.log.header[4] = 1u;
     a.log.header[5] = a.perm ? 1u : 0u;
+    a.log.header[9] = a.log.layout();
     if (!a.n_live) {
       a.log.header[6] = (uint32_t)(n_live & 0xFFFFFFFFll);
       a.log.header[7] = (uint32_t)(n_live >> 32);
@@ -837,15 +838,17 @@ cudaError_t launch_render_edit(int KP, int DEG, DType dt, const FwdArgs &a, cons
 // packet's chunks that hold a leaf and name its lane, in slot order, nseg[i]
 // of them.  count[i] = -1 when the ray's packet is not in the log (no log, a log
 // of other rays, or a packet that did not fit); chunk links are checked
-// against the log's size.
-__global__ void __launch_bounds__(256) log_read_kernel(const SampleLog l, long long n, const int *nseg, int max_out,
-                                                        int *leaf, float *chord, int *count) {
+// against the log's size.  packed, wide: the two views of the buffer, of which
+// the header names the one the forward wrote.
+__global__ void __launch_bounds__(256) log_read_kernel(const SampleLog packed, const SampleLog wide, long long n,
+                                                        const int *nseg, int max_out, int *leaf, float *chord,
+                                                        int *count) {
   const long long pos = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (pos >= n) return;
   int c = -1;
-  const bool valid = l.n_chunks && __ldg(l.header + 4) == 1u && __ldg(l.header) == l.n_chunks &&
-                     __ldg(l.header + 1) == (uint32_t)kLogRounds &&
-                     __ldg(l.header + 2) == (uint32_t)(n & 0xFFFFFFFFll) && __ldg(l.header + 3) == (uint32_t)(n >> 32);
+  const bool is_wide = wide.n_chunks && __ldg(wide.header + 9) == wide.layout();
+  const SampleLog &l = is_wide ? wide : packed;
+  const bool valid = l.n_chunks && log_matches(l, n);
   // the ray at this position (its outputs are written at the ray's index)
   const long long i = valid && __ldg(l.header + 5) == 1u ? (long long)min(__ldg(l.perm + pos), (uint32_t)(n - 1)) : pos;
   if (valid) {
@@ -862,10 +865,10 @@ __global__ void __launch_bounds__(256) log_read_kernel(const SampleLog l, long l
         }
         for (int k = 0; k < kLogRounds * 32 && c < want; ++k) {
           const size_t slot = (size_t)chunk * kLogRounds * 32 + k;
-          const uint32_t lf = __ldg(l.leaf + slot);
-          if (lf == kEmpty || __ldg(l.lane + slot) != (pos & 31)) continue;
+          const LogWord w = log_word(l, slot);
+          if (w.empty || w.lane != (int)(pos & 31)) continue;
           if (c < max_out) {
-            leaf[i * max_out + c] = (int)lf;
+            leaf[i * max_out + c] = (int)w.leaf;
             chord[i * max_out + c] = __ldg(l.dt + slot);
           }
           ++c;
@@ -881,10 +884,11 @@ __global__ void __launch_bounds__(256) log_read_kernel(const SampleLog l, long l
   count[i] = c;
 }
 
-cudaError_t launch_log_read(const SampleLog &l, long long n_rays, const int *nseg, int max_out, int *leaf,
-                            float *chord, int *count, cudaStream_t s) {
+cudaError_t launch_log_read(const SampleLog &packed, const SampleLog &wide, long long n_rays, const int *nseg,
+                            int max_out, int *leaf, float *chord, int *count, cudaStream_t s) {
   if (n_rays == 0) return cudaSuccess;
-  log_read_kernel<<<(unsigned)((n_rays + 255) / 256), 256, 0, s>>>(l, n_rays, nseg, max_out, leaf, chord, count);
+  log_read_kernel<<<(unsigned)((n_rays + 255) / 256), 256, 0, s>>>(packed, wide, n_rays, nseg, max_out, leaf,
+                                                                  chord, count);
   return cudaGetLastError();
 }
 
