@@ -81,7 +81,7 @@ struct neuvv_tree {
   uint32_t *child = nullptr;
   uint32_t *bricks = nullptr;
   uint32_t *coarse = nullptr;
-  uint32_t *queue = nullptr;   // triage of the packet forward: [kQueueEntries] (trees with a brick map)
+  uint32_t *queue = nullptr;   // triage of the packet forward: [kQueueEntries] (trees that gain from it)
   int brick_level = 0, brick_first = 0, brick_count = 0;
   void *rec = nullptr;
   float *master = nullptr, *m = nullptr, *v = nullptr;
@@ -680,10 +680,15 @@ neuvv_status neuvv_tree_create(const neuvv_tree_desc *desc, neuvv_tree **out) {
         for (size_t q = 0; q < n3; ++q) occ[q] = (map[q] >> 28) != kCoarseEmpty;
         const std::vector<int32_t> dist = chebyshev_distance(occ, nc, nc);
         std::vector<uint32_t> boxed(br);
+        // finest cells in leaves: of each brick, and all of a coarser leaf's cells
+        int64_t filled = 0, covered = 0;
+        for (uint32_t v : br) filled += (v & kBrickEmpty) != kBrickEmpty;
+        for (uint32_t w : map) covered += (w >> 28) != 0 && (w >> 28) != kCoarseEmpty;
         brick_empty_boxes(br, boxed, map, nc, d.depth);
         br.swap(boxed);
         coarse_empty_boxes(occ, dist, nc, map);
-        NEUVV_TRY(cudaMalloc(&t->queue, kQueueEntries * 4), "cudaMalloc(packet queue)");
+        if (triage_gains(Lb, filled + 512 * covered, 512 * (count + covered)))
+          NEUVV_TRY(cudaMalloc(&t->queue, kQueueEntries * 4), "cudaMalloc(packet queue)");
         NEUVV_TRY(cudaMalloc(&t->coarse, n3 * 4), "cudaMalloc(brick map)");
         NEUVV_TRY(cudaMemcpy(t->coarse, map.data(), n3 * 4, cudaMemcpyHostToDevice), "copy brick map");
       }

@@ -400,13 +400,6 @@ cudaError_t launch_triage_rays(const DevTree &tr, const DevRays &rays, const Dev
 // 1.0: 600 / 299 / 709 / 801; 1.6: 605 / 341 / 718 / 848; without triage 612 /
 // 340 / 722 / 848.  All packets in halves: 713 / 315 / 788 / 819.
 constexpr float kLongShare = 0.4f;
-// Shallower trees have short rays: their packets end together, and the pass of
-// 20 us is a notable part of the call (depth 6, 1293 x 886: 112 us without it, 128
-// with).
-// Solids (bricks at least half full) end their rays near the surface, which the
-// estimate does not see: a depth-8 solid at 1293 x 886 took 424 us without the
-// triage and 574 with it.
-constexpr int kTriageLevel = 5;
 
 // Launches a packet forward of any shading.  Up to four packets per resident
 // warp: a plain grid without counter or triage, each packet in as many parts
@@ -446,8 +439,7 @@ static cudaError_t packet_launch(FwdArgs a, const LaunchCfg &cfg, cudaStream_t s
       if ((e = launch_triage_rays(a.tr, a.rays, a.out, a.log.perm, a.log.perm, a.log.header + 6, a.log.header + 8, s)) !=
           cudaSuccess)
         return e;
-    } else if (!a.log.n_chunks && a.queue && a.tr.coarse && a.tr.brick_level >= kTriageLevel &&
-               2 * a.tr.n_leaves < ((long long)a.tr.brick_count << (3 * kBrickShift)) && n_packets <= kQueuePackets) {
+    } else if (!a.log.n_chunks && a.queue && n_packets <= kQueuePackets) {
       // a packet is long when its work is a notable part of an average warp's
       // share, which grows with the packets per resident warp
       uint32_t *counts = reinterpret_cast<uint32_t *>(a.work + 1);
