@@ -122,17 +122,16 @@ __global__ void __launch_bounds__(kGradTileW *kGradTileH)
 // One warp per word of the touched bitmap (32 leaves): an empty word is
 // skipped at once.  A group of kGroup lanes takes a leaf, a lane a 4-float quad
 // of its record, so a row is one coalesced access (half a warp where 16 lanes
-// cover the record); each group loads two rows of gradient, master and moments
-// before it updates either.  DRAM bound: 4.8 of the measured 6.78 TB/s with
-// one row at a time by a whole warp (K_pad 8: 15 of 32 lanes at work).
-template <int kGroup>
+// cover the record) and loads kRows rows of gradient, master and moments before
+// it updates them.  DRAM bound: 4.8 of the measured 6.78 TB/s with one row at a
+// time by a whole warp (K_pad 8: 15 of 32 lanes at work).
+template <int kGroup, int kRows>
 __global__ void __launch_bounds__(256) adam_kernel(float *__restrict__ master, float *__restrict__ m,
                                                    float *__restrict__ v, void *__restrict__ storage, int dt,
                                                    int storage_stride, float *__restrict__ grad,
                                                    const unsigned int *__restrict__ touched, long long n_leaves,
                                                    int stride_f32, int rec_len, float lr, float b1, float b2,
                                                    float eps, float c1, float c2) {
-  constexpr int kRows = 2;
   const int quads = (rec_len + 3) / 4;  // quads past the record's entries are padding and stay zero
   const int lane = threadIdx.x & 31, group = lane / kGroup, q0 = lane % kGroup;
   const float lr_c1 = lr / c1, inv_c2 = 1.f / c2;
@@ -353,12 +352,18 @@ cudaError_t launch_adam(float *master, float *m, float *v, void *storage, DType 
   }
   const long long want = ((n_leaves + 31) / 32 * 32 + 255) / 256;  // one warp per bitmap word
   const int blocks = (int)(want < 152 * 16 ? want : 152 * 16);
-  if (rec_len <= 64)
-    adam_kernel<16><<<blocks, 256, 0, s>>>(master, m, v, storage, (int)dt, storage_stride, grad, touched, n_leaves,
-                                           stride_f32, rec_len, lr, b1, b2, eps, c1, c2);
-  else
-    adam_kernel<32><<<blocks, 256, 0, s>>>(master, m, v, storage, (int)dt, storage_stride, grad, touched, n_leaves,
-                                           stride_f32, rec_len, lr, b1, b2, eps, c1, c2);
+  // Half warps with two rows each for records that 16 lanes cover.  A second row
+  // for a whole warp costs registers (48 -> 70) and so warps, and pays only where
+  // the record fills the warp.  Step over all leaves of a depth-7 solid (160,000) /
+  // depth-8 shell (500,000), us, two rows against one: K_pad 8 degree 2 (58 entries)
+  // 71 / 165 against 82 / 177; K_pad 16 degree 3 (122) 137 / 363 against 139 / 373;
+  // K_pad 16 degree 2 (74) 96 / 240 against 83 / 223; K_pad 8 degree 3 (106) 113 / 294
+  // against 106 / 289; K_pad 32 degree 3 (154) 174 / 450 against 150 / 431.
+  const auto kernel = rec_len <= 64                     ? adam_kernel<16, 2>
+                      : rec_len > 112 && rec_len <= 128 ? adam_kernel<32, 2>
+                                                        : adam_kernel<32, 1>;
+  kernel<<<blocks, 256, 0, s>>>(master, m, v, storage, (int)dt, storage_stride, grad, touched, n_leaves, stride_f32,
+                                rec_len, lr, b1, b2, eps, c1, c2);
   return cudaGetLastError();
 }
 
