@@ -3,8 +3,8 @@
 // render_plain_kernel  : one thread per ray, child table read from global
 //                        memory -- the baseline single-view path.
 // render_packet_kernel : one thread per ray with warps as 32-ray packets;
-//                        walking and shading decoupled through a per-lane
-//                        queue of found segments; descents restart at the
+//                        walking and shading decoupled through one ring of
+//                        found segments per packet; descents restart at the
 //                        lowest common ancestor of successive cells.
 #include "neuvv_kernels.h"
 #include "neuvv_ray.cuh"
@@ -401,14 +401,17 @@ cudaError_t launch_triage_rays(const DevTree &tr, const DevRays &rays, const Dev
 // 340 / 722 / 848.  All packets in halves: 713 / 315 / 788 / 819.
 constexpr float kLongShare = 0.4f;
 
-// Launches a packet forward of any shading.  Up to four packets per resident
-// warp: a plain grid without counter or triage, each packet in as many parts
-// (up to four) as keep to that number, since these calls are bound by the
-// latency of their longest packet (a 128 x 128 view: 78 us whole, 49 in four
-// parts; without a log, whose layout is by whole packets).  Above: a persistent grid on the work counter, after the triage
-// that the call allows: of rays with a log in which the packets are taken as
-// given (n < 2^32), of packets without a log on trees of depth 8 to 10 (with a
-// brick map) whose bricks are less than half full.
+// Launches a packet forward of any shading.  Without a log each packet is run
+// in two or four parts while the parts stay within four per resident warp (up
+// to two packets per warp in halves, up to one in quarters), on a plain grid without
+// counter or triage: these calls are bound by the latency of their longest
+// packet (a 128 x 128 view: 78 us whole, 49 in four parts).  A log's layout is by
+// whole packets, so calls with one run them whole, on a plain grid up to one
+// packet per resident warp.  Above: a persistent grid on the work counter, after
+// the triage that the call allows: of rays with a log in which the packets are
+// taken as given (n < 2^32), of packets without a log on the trees that gain from
+// it (triage_gains; already at 2.5 packets per warp: a 480 x 400 view of a depth-8
+// shell 189 us with the list, 273 without).
 template <int KP, int DEG, typename E, int kShade, int CHUNKS = shade_chunks<KP, DEG, E, kShade>()>
 static cudaError_t packet_launch(FwdArgs a, const LaunchCfg &cfg, cudaStream_t s) {
   if (a.rays.n == 0) return cudaSuccess;
