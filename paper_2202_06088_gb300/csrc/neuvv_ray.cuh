@@ -165,13 +165,15 @@ struct PacketShared {
   }
   __device__ __forceinline__ SmemRows<KP> rows_of(int lane) const { return SmemRows<KP>{rows + lane, stride}; }
   // Entries of the batch that belong to this lane's ray, as a mask (entry j
-  // of `owner` in lane j when has).
+  // of `owner` in lane j when has).  Collected with shared-memory atomics: a
+  // match over the warp took some 5 % of a call whose packets are coherent (1080p
+  // view of a depth-7 solid, K_pad 8 BF16, 1.02 -> 0.95 of the time with a queue per
+  // ray; density alone 1.05 -> 0.91; depth-8 shell 0.85 -> 0.82).
   __device__ __forceinline__ unsigned entries_of_lane(bool has, int owner) const {
     const int lane = threadIdx.x & 31;
-    const unsigned grp = __match_any_sync(kFull, has ? owner : 32 + lane);
     own[lane] = 0u;
     __syncwarp();
-    if (has && lane == __ffs(grp) - 1) own[owner] = grp;
+    if (has) atomicOr(own + owner, 1u << lane);
     __syncwarp();
     return own[lane];
   }
