@@ -1124,19 +1124,18 @@ neuvv_status prepare_compose(const neuvv_tree *const *trees, const float *transf
       }
     for (int r = 0; r < 3; ++r) p.trans[r] = (float)tr[r];
     p.scale = (float)std::sqrt(s2);
-    // a ball that holds the box, its centre relative to the translation: 1e-3
-    // of the radius and 2^-20 of the offset are above what FP32 rounds off the
-    // offset, the transform and the sums that use them
-    double r2 = 0.0, off2 = 0.0;
+    // a ball that holds the box: 1e-3 of the radius is above what FP32 rounds off
+    // the transform, 2^-22 of the centre above what it rounds off the centre
+    double r2 = 0.0, centre2 = 0.0;
     for (int r = 0; r < 3; ++r) {
-      double c = 0.0;
+      double c = tr[r];
       for (int k = 0; k < 3; ++k) c += m[r][k] * 0.5 * ((double)t->bmin[k] + (double)t->bmax[k]);
       p.ball[r] = (float)c;
-      off2 += c * c;
+      centre2 += c * c;
       const double half = 0.5 * ((double)t->bmax[r] - (double)t->bmin[r]);
       r2 += s2 * half * half;
     }
-    const double radius = 1.001 * std::sqrt(r2) + std::ldexp(std::sqrt(off2), -20);
+    const double radius = 1.001 * std::sqrt(r2) + std::ldexp(std::sqrt(centre2), -22);
     p.ball[3] = (float)(radius * radius);
     if (!std::isfinite(time_offsets[j])) return fail(NEUVV_ERR_INVALID_ARG, "time offset %d not finite", j);
     p.toff = time_offsets[j];

@@ -158,18 +158,15 @@ __device__ __forceinline__ bool walk_init_local(const DevTree &tr, const PrimPar
 
 // Whether the line o + s d can reach the ball around a primitive's box: the
 // cheap test that most (ray, primitive) pairs end at.  No pair that the exact
-// test accepts is lost.  The ball's centre is kept as an offset from the
-// translation, which is subtracted from the ray's origin first (exact when they
-// are close), and the radius holds the offset's rounding (prepare_compose), so
-// a small primitive far from the world's origin keeps its corners; 1e-5 of the
-// squared distance is far above the FP32 error of the expression.  id:
-// 1 / |d|, or NaN where its square leaves the FP32 range: a comparison with
-// NaN accepts.
-__device__ __forceinline__ bool near_ball(const PrimParam &pp, const float o[3], const float d[3], float id) {
-  const float m0 = (pp.trans[0] - o[0]) + pp.ball[0], m1 = (pp.trans[1] - o[1]) + pp.ball[1],
-              m2 = (pp.trans[2] - o[2]) + pp.ball[2];
-  const float mm = fmaf(m0, m0, fmaf(m1, m1, m2 * m2)), md = fmaf(m0, d[0], fmaf(m1, d[1], m2 * d[2])) * id;
-  return !(mm - md * md > fmaf(1e-5f, mm, pp.ball[3]));
+// test accepts is lost: the radius holds the rounding of the ball's centre
+// (prepare_compose), which far from the world's origin is a sizeable part of a
+// small ball, and 1e-5 of the squared distance is far above the FP32 error of the
+// expression.  idd: 1 / |d|^2; taken between the two factors, short directions
+// do not underflow, and where it is infinite the comparison accepts.
+__device__ __forceinline__ bool near_ball(const PrimParam &pp, const float o[3], const float d[3], float idd) {
+  const float m0 = pp.ball[0] - o[0], m1 = pp.ball[1] - o[1], m2 = pp.ball[2] - o[2];
+  const float mm = fmaf(m0, m0, fmaf(m1, m1, m2 * m2)), md = fmaf(m0, d[0], fmaf(m1, d[1], m2 * d[2]));
+  return !(fmaf(-md * idd, md, mm) > fmaf(1e-5f, mm, pp.ball[3]));
 }
 
 // One packet of 32 rays per warp.  The primitives are taken one after another
@@ -205,13 +202,12 @@ __global__ void __launch_bounds__(256, packet_min_blocks<KP, DEG, E>())
     const bool live = i < n;
     float o[3] = {0.f, 0.f, 0.f}, d[3] = {0.f, 0.f, 0.f}, t = 0.f;
     if (live) load_ray(a.rays, i, o, d, t);
-    const float dd = fmaf(d[0], d[0], fmaf(d[1], d[1], d[2] * d[2]));
-    const float id = dd > 1e-30f && dd < 1e30f ? 1.f / sqrtf(dd) : NAN;
+    const float idd = 1.f / fmaf(d[0], d[0], fmaf(d[1], d[1], d[2] * d[2]));
     float Lc[kMaxPrims][3], La[kMaxPrims], Ld[kMaxPrims];
     int n_layers = 0;
     for (int j = 0; j < a.n_prims; ++j) {
       const PrimParam &pp = a.prim[j];
-      const bool close = live && near_ball(pp, o, d, id);
+      const bool close = live && near_ball(pp, o, d, idd);
       if (!__any_sync(kFull, close)) continue;
       const DevTree &tr = a.trees[pp.tree];
       RayWalk w;

@@ -157,7 +157,7 @@ struct PrimParam {
   float minv_lo[9];  // ... and the remainders: minv + minv_lo is the inverse to ~2^-48
   float trans[3];    // translation of world-from-local
   float scale;     // s
-  float ball[4];   // centre of the box relative to trans and the square of a radius that holds the box
+  float ball[4];   // world centre of the box and the square of a radius that holds it
   float toff;      // time offset, frames
   float tint[3];
   int tree;        // index into ComposeArgs::trees
