@@ -175,8 +175,8 @@ __device__ __forceinline__ bool near_ball(const PrimParam &pp, const float o[3],
 // (shade_batch), and the ray's sums become a layer.  A ray that misses a
 // primitive leaves no layer (it would have colour and alpha 0 and an infinite
 // depth, which change neither blending mode).  Bound by issue and dependent
-// arithmetic (52 % of issue slots at 16 warps per SM).  8 primitives,
-// 2 x 2160^2: 1963 us with lockstep walking and shading per ray, 1046 now.
+// arithmetic (53 % of issue slots at 16 warps per SM).  8 primitives,
+// 2 x 2160^2: 1920 us with lockstep walking and shading per ray, 962 now.
 template <int KP, int DEG, typename E>
 __global__ void __launch_bounds__(256, packet_min_blocks<KP, DEG, E>())
     compose_kernel(const __grid_constant__ ComposeArgs a, int dynamic) {

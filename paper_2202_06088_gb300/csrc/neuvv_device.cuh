@@ -114,7 +114,7 @@ __device__ __forceinline__ void raise_status(const DevTree &tr, uint32_t bit) {
 // reduced by 1.5 * 2^23 is its exact FP32 value, and the floor of p is the
 // bits of p + 1.5 * 2^23 rounded down: no conversion instruction in the step.
 // One 1080p view of a depth-9 shell (2 M leaves, BF16): 311 -> 270 M warp
-// instructions, 763 -> 671 us, outputs bit for bit those of the walk before.
+// instructions, 763 -> 671 us, segments bit for bit those of the walk before.
 // ---------------------------------------------------------------------------
 constexpr int kMagicBits = 0x4B400000;      // 1.5 * 2^23 as bits ...
 constexpr float kMagic = 12582912.f;        // ... and as a value (|cell| < 2^22)
@@ -860,7 +860,7 @@ struct Sample {
 // Where a ray's interpolated basis rows a(u), b(u) live, in quads: registers
 // (RegRows) or a column of shared memory (SmemRows: value k at p[k * stride], b
 // after a; lanes read the columns of any rays without bank conflicts, which
-// rows of quads at an odd pitch did not: 3.12 against 2.94 ms for the replay
+// rows of quads at an odd pitch did not: 3.12 against 3.03 ms for the replay
 // of the 8-view step).
 template <int KP>
 struct RegRows {

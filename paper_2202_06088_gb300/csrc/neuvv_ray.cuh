@@ -66,9 +66,9 @@ __device__ __forceinline__ void integrate_ray(const DevTree &tr, const float o[3
 // six hundred instructions, and packets of uneven or incoherent rays would
 // run them with few lanes active if each lane shaded its own ray's segments
 // only -- and each ray then composites its own entries of the batch in order.
-// Against a queue per ray (lanes active per instruction): 1080p view 21.7 ->
-// 28.5 of 32, 671 -> 658 us; 262,144 rays in drawn order 5.2 -> 9.9, training
-// step 3.15 -> 1.38 ms.
+// Against a queue per ray, lanes active per instruction, walk included: 1080p view
+// 21.7 -> 26.6 of 32; 262,144 rays in drawn order 5.2 -> 13.2 in the forward and
+// 5.7 -> 25.4 in the adjoint, training step 3.25 -> 1.24 ms.
 // ---------------------------------------------------------------------------
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
@@ -128,7 +128,7 @@ struct PacketShared {
   // entries) into the staging area.  A group of kGroup lanes takes one record,
   // a lane a chunk, so a warp's load covers whole lines (each lane reading its
   // own record 16 bytes at a time touches 32 lines per load; those wavefronts
-  // kept L1 at 56 % of its peak in the 1080p forward, against 19 % now).  The
+  // kept L1 at 56 % of its peak in the 1080p forward, against 18 % now).  The
   // copies run while the rays walk on.  Lanes without an entry pass leaf 0.
   static constexpr int kGroup = CHUNKS > 16 ? 32 : (CHUNKS > 8 ? 16 : 8);
   __device__ __forceinline__ void stage_records(const void *base, uint32_t rec_bytes, uint32_t leaf, int count) const {

@@ -394,11 +394,11 @@ cudaError_t launch_triage_rays(const DevTree &tr, const DevRays &rays, const Dev
 }
 
 // Bricks per ray, per packet of a resident warp's share, from which a packet
-// counts as long (see packet_launch).  Measured us of a 1080p view / an FP8 view
-// of 1283 x 717 / a slice and its 1080p view / an edited 720p frame: 0.25:
-// 612 / 317 / 728 / 812; 0.4: 571 / 285 / 693 / 795; 0.65: 588 / 285 / 708 / 804;
-// 1.0: 600 / 299 / 709 / 801; 1.6: 605 / 341 / 718 / 848; without triage 612 /
-// 340 / 722 / 848.  All packets in halves: 713 / 315 / 788 / 819.
+// counts as long (see packet_launch).  Measured us, caches flushed between passes,
+// of a 1080p view / an FP8 view of 1283 x 717 / a slice and its 1080p view / an
+// edited 720p frame: 0.25: 598 / 335 / 724 / 594; 0.4: 570 / 305 / 668 / 561; 0.65:
+// 622 / 299 / 727 / 564; 1.0: 665 / 307 / 754 / 585; without triage 658 / 415 / 752 /
+// 665.
 constexpr float kLongShare = 0.4f;
 
 // Launches a packet forward of any shading.  Without a log each packet is run
